@@ -17,6 +17,7 @@
 
 #include "../../include/sssp.h"
 #include "cluster_launch.h"
+#include "eo_launch.h"
 #include "march_kernel.cuh"
 #include "march_large.cuh"
 #include "fd_launch.h"
@@ -122,8 +123,11 @@ cudaError_t set_smem_attr() {
   if (done_dev == dev) return cudaSuccess;
   const int sm = int(Cfg<LOG2L>::SMEM), smc = int(Cfg<LOG2L>::SMEM_CPLX);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet>, a, smc);
+  cudaError_t e = cudaSuccess;
+  if constexpr (LOG2L < sssp_eo::kMinLog2) {
+    e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet>, a, smc);
+  }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic>, a, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic>, a, smc);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet>, a, sm);
@@ -144,7 +148,7 @@ cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTa
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
       sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<count, nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
-  } else {
+  } else if constexpr (LOG2L < sssp_eo::kMinLog2) {
     if (cplx)
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
@@ -245,6 +249,10 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
     if (bc != sssp::kBcDirichlet) return cudaErrorInvalidValue;
     return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx);
   }
+  // Dirichlet, L >= 512: the parity-split kernel, faster at every count there (one solve of L = 1024
+  // 2250 -> 1720 cycles a transform, two an SM 3550 -> 2410, one of L = 2048 4600 -> 3040, of L = 4096
+  // 6900 -> 6050); below it the half-transforms have fewer points than a warp's eight per lane
+  if (bc == sssp::kBcDirichlet && sssp_eo::supported(log2L)) return sssp_eo::launch_march(log2L, d, count, st, cplx);
   switch (log2L) {
     case 3: return launch_march_t<3>(d, count, tabs, st, cplx, bc);
     case 4: return launch_march_t<4>(d, count, tabs, st, cplx, bc);
@@ -626,6 +634,8 @@ pe_status pe_plan_create_bc(pe_plan** out, int N, double H, double k0, double dr
   if (e != cudaSuccess) return bail(e, "cudaGetDevice");
   e = get_tables(p->device, log2L, &p->tabs);
   if (e != cudaSuccess) return bail(e, "transform tables");
+  if (bc == PE_BC_DIRICHLET && sssp_eo::supported(log2L) && (e = sssp_eo::prepare(log2L)) != cudaSuccess)
+    return bail(e, "parity-split kernel tables");
   // plan tables in FP64 (Section 3: 1/(1 + b_j lambda_m), lambda_m = -(pi m/(k0 H))^2)
   const int L = p->L, P = pade_order;
   std::vector<float4> R(size_t(P) * L), G(L);

@@ -1382,3 +1382,38 @@ def test_fdssp_range_dependent_nodes(sssp):
     tl, _ = pl.read_tl()
     pl.close()
     _compare(u, tl, _fd_oracle(s, 25))
+
+
+# ----------------------------------------------------------------------------- parity-split one-CTA kernel
+@pytest.mark.parametrize("N", [511, 1023, 2047, 4095])
+@pytest.mark.parametrize("terms,absorb", [(1, False), (2, False), (5, False), (12, True)])
+def test_parity_split_march_against_oracle(sssp, N, terms, absorb):
+    """The one-CTA kernel with the modes split by parity, at every size it takes (each has its own
+    middle radix 4, 8, 16 or 32), for series of one term (V ignored), two (the loop's shortest), five
+    and the full rule, real and complex profiles, a node change half way, and a TL row every step,
+    from a field on every depth point (so every mode and both extra points M/2 carry weight).
+    Bound: a transform's FP32 error is below 1e-6 log2 L of its input, 3 steps of [4/4] chain at
+    most 12 stages whose corrections are below half the field, each through two transforms."""
+    s = inputs.munk(N=N, freq=0.06 * (N + 1), dr=50.0 if N < 1000 else 25.0, steps=3, pade_order=4, neumann_terms=terms)
+    rng = np.random.default_rng(N + terms)
+    n = np.arange(1, N + 1)
+    a = (rng.standard_normal(N) + 1j * rng.standard_normal(N)) / (1.0 + 8.0 * n / N) ** 2
+    s.u0 = O.idst1(a) * N ** 0.5
+    n2 = s.profiles[0][1]
+    other = 1.0 + 0.9 * (n2 - 1.0) + 0.002 * np.sin(3.0 * np.pi * s.z / s.H)
+    if absorb:
+        other = other + 0.001j * (s.z / s.H) ** 2
+    s.profiles = [(0.0, n2.astype(other.dtype)), (1.5 * s.dr, other)]
+    pl = sssp.plan_for(s, tl_every=1)
+    pl.set_kernel("cta")
+    assert pl.shape == 8
+    pl.march(s.steps)
+    u, (tl, _) = pl.read_field(), pl.read_tl()
+    pl.close()
+    if terms == 1:
+        s.profiles = [(0.0, np.ones(N))]
+    ref = _oracle(s)
+    assert np.linalg.norm(u - ref.u) / np.linalg.norm(ref.u) <= 12e-6 * math.log2(N + 1) / 8
+    for k in range(s.steps):  # the rows as magnitudes: every depth point, weighted by its own size
+        got, want = 10.0 ** (-tl[k].astype(np.float64) / 20.0), 10.0 ** (-ref.tl[k] / 20.0)
+        assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 12e-6 * math.log2(N + 1) / 8
