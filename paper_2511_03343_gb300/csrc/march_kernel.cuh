@@ -823,13 +823,28 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
   }
 }
 
+// What setting a starter does beside its transform: the physical field as given (index 0 the zero
+// boundary on Dirichlet grids) and a cleared status word.  Null in the transform entry points.
+struct StartArgs {
+  float2* field = nullptr;
+  int* status = nullptr;
+  int mirror = 0;  // K > 0: in holds K + 1 values and the grid is their even extension to 2 K points
+};
+
+// Point n of the grid, from the caller's values (Dirichlet: N interior points; periodic: all points)
+template <int BC>
+__device__ __forceinline__ float2 start_value(const float2* in, int n, int mirror) {
+  if constexpr (BC == kBcPeriodic) return in[mirror > 0 && n > mirror ? 2 * mirror - n : n];
+  else return n == 0 ? make_float2(0.f, 0.f) : in[n - 1];
+}
+
 // DST-I of one field per CTA: out = scale * DST(in); field b = blockIdx.x reads N values at
 // in + b * in_stride (n = 1..N) and writes L values at out + b * out_stride.
 template <int LOG2L, int BC = kBcDirichlet>
 __global__ void __launch_bounds__(Cfg<LOG2L>::NT)
     sssp_dst_kernel(const float2* __restrict__ in, float2* __restrict__ out, float scale,
-                    const float2* __restrict__ tw_g, const float* __restrict__ sin_g, long long in_stride = 0,
-                    long long out_stride = 0) {
+                    const float2* __restrict__ tw_g, const float* __restrict__ sin_g, long long in_stride,
+                    long long out_stride, const StartArgs sa) {
   using C = Cfg<LOG2L>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem<LOG2L> sm(smem_raw);
@@ -837,14 +852,30 @@ __global__ void __launch_bounds__(Cfg<LOG2L>::NT)
   in += blockIdx.x * in_stride;
   out += blockIdx.x * out_stride;
   load_tables<LOG2L>(sm.tw, sm.sinw, tw_g, sin_g);
-  for (int n = t; n < C::L; n += C::NT)
-    sm.bufA[pidx(n)] = (BC == kBcPeriodic) ? in[n] : ((n == 0) ? make_float2(0.f, 0.f) : in[n - 1]);
+  for (int n = t; n < C::L; n += C::NT) {
+    const float2 v = start_value<BC>(in, n, sa.mirror);
+    sm.bufA[pidx(n)] = v;
+    if (sa.field) sa.field[n] = v;
+  }
+  if (sa.status && t == 0) *sa.status = kStatusOk;
   __syncthreads();
   float2 o[8];
   xform<LOG2L, BC, false>(sm.bufA, sm.bufB, sm.tw, sm.sinw, sm.scan_s, o);
 #pragma unroll
   for (int i = 0; i < 8; ++i) o[i] = scale * o[i];
   store8<LOG2L>(out + 8 * t, o);
+}
+
+// The same without a transform (grids whose transform is another kernel; FD-SSP plans, which march
+// depth values: state = field)
+template <int BC>
+__global__ void sssp_start_kernel(const float2* __restrict__ in, float2* __restrict__ state, int L, const StartArgs sa) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n == 0) *sa.status = kStatusOk;
+  if (n >= L) return;
+  const float2 v = start_value<BC>(in, n, sa.mirror);
+  sa.field[n] = v;
+  if (state) state[n] = v;
 }
 
 }  // namespace sssp

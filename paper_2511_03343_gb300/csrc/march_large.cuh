@@ -84,6 +84,8 @@ struct BigCfg {
   static constexpr int TILE = kLargeTile;
   static constexpr int LOG2TC = kLargeLog2Tile - LOG2P, LOG2TR = kLargeLog2Tile - LOG2Q;
   static constexpr int TC = 1 << LOG2TC, TR = 1 << LOG2TR;  // columns / rows per tile
+  static constexpr int NA = (Q / 2) / TC + 1;   // pass-A tiles; the last ends at column Q/2 (overlap rewrites)
+  static constexpr int NBT = (P / 2) / TR + 1;  // pass-B tiles; the last ends at row P/2 (its other rows: done)
   static constexpr int RSP = P + P / 16 + 1, RSQ = Q + Q / 16 + 1;  // padded FFT strides
   static constexpr int BUF = (TC * RSP > TR * RSQ) ? TC * RSP : TR * RSQ;
   // pass A's twiddles w_{2L}^e, e = col k1 < L, as the product of two table entries
@@ -162,29 +164,20 @@ __device__ __forceinline__ void load_large_twiddles(float2* sm, const LargeTabs&
   for (int i = threadIdx.x; i < C::Q / 2; i += kLargeNT) tq[i] = tb.tw2L[C::P * i];
 }
 
-// Unnormalised DST-I S_k = sum_n x_n sin(pi n k/L), k in [0, L) (S_0 = 0), of the values the
-// source gives: src(m, first) returns x_m (m in [1, L)); it is called twice per m in pass A (for
-// z_m and z_{2L-m}), `first` true on the first.  The sink takes snk(k, S_k) once per k in pass B.
-// Pass A reads every source value before pass B writes anything, so a source and sink may share
-// an array (in-place transform).  W: 2L scratch.  On return all threads are past a barrier.
-template <int LOG2L, class SRC, class SNK>
-__device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC& src, SNK& snk) {
+// pass A on the tiles [c0, c1): the P-point FFTs of the stored columns n2 in [0, Q/2], twiddled, into
+// W[k1][n2]
+template <int LOG2L, class SRC>
+__device__ __forceinline__ void dst_pass_a(float2* W, float2* sm, const SRC& src, int c0, int c1) {
   using C = BigCfg<LOG2L>;
   constexpr int L = C::L, P = C::P, Q = C::Q, QH = Q / 2, QS = QH + 1;
-  constexpr int TC = C::TC, TR = C::TR;
-  constexpr int LOG2QH = C::LOG2Q - 1;
-  constexpr int NA = QH / TC + 1;  // pass-A tiles; the last ends at column Q/2 (overlap rewrites)
+  constexpr int TC = C::TC, NA = C::NA, PT = kLargePT;
   const int t = threadIdx.x;
   float2* bufA = sm;
   float2* bufB = sm + C::BUF;
   const float4* twP = reinterpret_cast<const float4*>(sm + 2 * C::BUF);  // copied by load_large_twiddles
-  const float4* twQ = twP + P;
-  const float4* tlo = twQ + Q;
+  const float4* tlo = twP + P + Q;
   const float4* thi = tlo + C::R;
-  const float4* tq = thi + C::NT1;
-  constexpr int PT = kLargePT, PH = kLargePT / 2;
-  float2 pre[PT + 1];
-  // pass A: the P-point FFTs of the stored columns n2 in [0, Q/2], twiddled, into W[k1][n2]
+  float2 pre[PT];
   auto loadA = [&](int c) {
     const int cb = c < NA - 1 ? c * TC : QH - TC + 1;
 #pragma unroll
@@ -217,9 +210,9 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
     src.l2(lo < 1 ? 1 : lo);
     src.l2(hi > L - 1 ? L - 1 : hi);
   };
-  if (NA > 1) l2A(1);
-  loadA(0);
-  for (int c = 0; c < NA; ++c) {
+  if (c0 + 1 < c1) l2A(c0 + 1);
+  loadA(c0);
+  for (int c = c0; c < c1; ++c) {
     const int cb = c < NA - 1 ? c * TC : QH - TC + 1;
 #pragma unroll
     for (int q = 0; q < PT; ++q) {
@@ -227,8 +220,8 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
       bufA[(idx & (TC - 1)) * C::RSP + pidx(idx >> C::LOG2TC)] = pre[q];
     }
     __syncthreads();
-    if (c + 1 < NA) loadA(c + 1);
-    if (c + 2 < NA) l2A(c + 2);
+    if (c + 1 < c1) loadA(c + 1);
+    if (c + 2 < c1) l2A(c + 2);
     const float2* F = tfft<C::LOG2P, C::RSP, 1>(bufA, bufB, twP);
 #pragma unroll
     for (int q = 0; q < PT; ++q) {
@@ -240,12 +233,25 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
     }
     __syncthreads();
   }
-  // pass B: the rows k in [0, P/2].  The odd symmetry of z gives the unstored half of a row from
-  // its partner row P - k: Y[k][Q - n] = -w_Q^{-n} Y[P - k][n] (k != 0), -Y[0][n] (k = 0).  A row's
-  // Q outputs are Z_{k + P k2}; those with k + P k2 >= L are -Z at 2L - k - P k2 = (P - k) +
-  // P (Q - 1 - k2), the partner row's, so one FFT per row pair yields both rows' S values
-  // (rows 0 and P/2 are their own partners: only their first Q/2 outputs are kept).
-  constexpr int NBT = (P / 2) / TR + 1;  // the last tile ends at row P/2 (its other rows: done)
+}
+
+// pass B on the tiles [t0, t1): the rows k in [0, P/2].  The odd symmetry of z gives the unstored half
+// of a row from its partner row P - k: Y[k][Q - n] = -w_Q^{-n} Y[P - k][n] (k != 0), -Y[0][n] (k = 0).
+// A row's Q outputs are Z_{k + P k2}; those with k + P k2 >= L are -Z at 2L - k - P k2 = (P - k) +
+// P (Q - 1 - k2), the partner row's, so one FFT per row pair yields both rows' S values
+// (rows 0 and P/2 are their own partners: only their first Q/2 outputs are kept).
+template <int LOG2L, class SNK>
+__device__ __forceinline__ void dst_pass_b(const float2* W, float2* sm, SNK& snk, int t0, int t1) {
+  using C = BigCfg<LOG2L>;
+  constexpr int L = C::L, P = C::P, Q = C::Q, QH = Q / 2, QS = QH + 1;
+  constexpr int TR = C::TR, NBT = C::NBT, LOG2QH = C::LOG2Q - 1;
+  constexpr int PT = kLargePT, PH = kLargePT / 2;
+  const int t = threadIdx.x;
+  float2* bufA = sm;
+  float2* bufB = sm + C::BUF;
+  const float4* twQ = reinterpret_cast<const float4*>(sm + 2 * C::BUF) + P;
+  const float4* tq = twQ + Q + C::R + C::NT1;
+  float2 pre[PT + 1];
   auto rowof = [&](int tile, int sl) { return (tile < NBT - 1 ? tile * TR : P / 2 - TR + 1) + sl; };
   auto l2B = [&](int tile) {  // the lines of a tile's sink operands, one per thread
     constexpr int LPK = TR / 16;          // lines per output column k2 and side
@@ -263,7 +269,7 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
     snk.l2(lo < 0 ? 0 : lo);
     snk.l2(hi > L - 1 ? L - 1 : hi);
   };
-  if (SNK::kL2) l2B(0);
+  if (SNK::kL2) l2B(t0);
   auto loadB = [&](int tile) {
 #pragma unroll
     for (int q = 0; q < PH; ++q) {  // own stored half, columns [0, Q/2)
@@ -294,8 +300,8 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
     neg = true;
     return true;
   };
-  loadB(0);
-  for (int tile = 0; tile < NBT; ++tile) {
+  loadB(t0);
+  for (int tile = t0; tile < t1; ++tile) {
 #pragma unroll
     for (int q = 0; q < PH; ++q) {
       const int idx = t + q * kLargeNT;
@@ -320,8 +326,8 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
       bool ng;
       if (target(tile, q, tg, ng)) snk.prefetch(q, tg);
     }
-    if (tile + 1 < NBT) loadB(tile + 1);
-    if (SNK::kL2 && tile + 1 < NBT) l2B(tile + 1);
+    if (tile + 1 < t1) loadB(tile + 1);
+    if (SNK::kL2 && tile + 1 < t1) l2B(tile + 1);
     const float2* F = tfft<C::LOG2Q, C::RSQ, 1>(bufA, bufB, twQ);
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
@@ -347,6 +353,17 @@ __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC
     }
     __syncthreads();
   }
+}
+
+// Unnormalised DST-I S_k = sum_n x_n sin(pi n k/L), k in [0, L) (S_0 = 0), of the values the
+// source gives: src(m, first) returns x_m (m in [1, L)); it is called twice per m in pass A (for
+// z_m and z_{2L-m}), `first` true on the first.  The sink takes snk(k, S_k) once per k in pass B.
+// Pass A reads every source value before pass B writes anything, so a source and sink may share
+// an array (in-place transform).  W: 2L scratch.  On return all threads are past a barrier.
+template <int LOG2L, class SRC, class SNK>
+__device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC& src, SNK& snk) {
+  dst_pass_a<LOG2L>(W, sm, src, 0, BigCfg<LOG2L>::NA);
+  dst_pass_b<LOG2L>(W, sm, snk, 0, BigCfg<LOG2L>::NBT);
 }
 
 // sources (depth or spectral values the transform reads) and sinks (where its outputs go)
@@ -585,6 +602,26 @@ __global__ void __launch_bounds__(kLargeNT, 1)
   __syncthreads();
   SnkScaled sk{out, scale};
   dst_global<LOG2L>(work, tb, tile_smem, SrcIn{in}, sk);
+}
+
+// The same transform with a CTA per tile, pass A and pass B as two launches (grid: tiles x fields): one
+// field on its own keeps one SM busy in the kernel above.  The tiles' arithmetic is the same, so the
+// results are too, bit for bit.
+template <int LOG2L, bool PASS_B>
+__global__ void __launch_bounds__(kLargeNT, 1)
+    sssp_dst_large_tile_kernel(const float2* in, float2* __restrict__ out, float scale, float2* work, const LargeTabs tb,
+                               long long in_stride, long long out_stride) {
+  extern __shared__ __align__(16) float2 tile_smem[];
+  work += blockIdx.y * (long long)large_work_elems(1 << LOG2L);
+  load_large_twiddles<LOG2L>(tile_smem, tb);
+  __syncthreads();
+  const int c = blockIdx.x;
+  if constexpr (PASS_B) {
+    SnkScaled sk{out + blockIdx.y * out_stride, scale};
+    dst_pass_b<LOG2L>(work, tile_smem, sk, c, c + 1);
+  } else {
+    dst_pass_a<LOG2L>(work, tile_smem, SrcIn{in + blockIdx.y * in_stride}, c, c + 1);
+  }
 }
 
 }  // namespace sssp

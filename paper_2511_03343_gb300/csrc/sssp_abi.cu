@@ -159,15 +159,16 @@ cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTa
 
 template <int LOG2L>
 cudaError_t launch_dst_t(const float2* in, float2* out, float scale, const TransformTables& tabs, cudaStream_t st,
-                         int count = 1, long long in_stride = 0, long long out_stride = 0, int bc = 0) {
+                         int count = 1, long long in_stride = 0, long long out_stride = 0, int bc = 0,
+                         const sssp::StartArgs& sa = {}) {
   cudaError_t e = set_smem_attr<LOG2L>();
   if (e != cudaSuccess) return e;
   if (bc == sssp::kBcPeriodic)
     sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
-        in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride);
+        in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
   else
     sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
-        in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride);
+        in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
   return cudaGetLastError();
 }
 
@@ -219,9 +220,16 @@ cudaError_t large_tabs(sssp::LargeTabs* out) {
   if ((e = cudaFuncSetAttribute(sssp::sssp_march_large_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 int(B::SMEM))) != cudaSuccess)
     return e;
-  return cudaFuncSetAttribute(sssp::sssp_dst_large_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(B::SMEM));
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if ((e = cudaFuncSetAttribute(sssp::sssp_dst_large_tile_kernel<LOG2L, false>, at, int(B::SMEM))) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(sssp::sssp_dst_large_tile_kernel<LOG2L, true>, at, int(B::SMEM))) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(sssp::sssp_dst_large_kernel<LOG2L>, at, int(B::SMEM));
 }
+
+// Fields up to which the large transform runs a CTA per tile.  Batched call at L = 65536, a CTA per field
+// against a CTA per tile: 1 field 113 / 29 us, 16 fields 122 / 41, 32 fields 132 / 61 (L = 16384: 32 fields
+// 48 / 32); the tiles' time grows with the fields once they fill the SMs, the other hardly before 64.
+constexpr int kLargeTileFields = 32;
 
 template <int LOG2L>
 cudaError_t launch_march_large_t(const SolveDesc* dDescs, int count, const TransformTables&, cudaStream_t st) {
@@ -238,8 +246,16 @@ cudaError_t launch_dst_large_t(const float2* in, float2* out, float scale, float
   sssp::LargeTabs tb;
   cudaError_t e = large_tabs<LOG2L>(&tb);
   if (e != cudaSuccess) return e;
-  sssp::sssp_dst_large_kernel<LOG2L><<<count, sssp::kLargeNT, sssp::BigCfg<LOG2L>::SMEM, st>>>(
-      in, out, scale, work, tb, in_stride, out_stride);
+  using B = sssp::BigCfg<LOG2L>;
+  if (count <= kLargeTileFields) {
+    sssp::sssp_dst_large_tile_kernel<LOG2L, false><<<dim3(B::NA, count), sssp::kLargeNT, B::SMEM, st>>>(
+        in, out, scale, work, tb, in_stride, out_stride);
+    sssp::sssp_dst_large_tile_kernel<LOG2L, true><<<dim3(B::NBT, count), sssp::kLargeNT, B::SMEM, st>>>(
+        in, out, scale, work, tb, in_stride, out_stride);
+  } else {
+    sssp::sssp_dst_large_kernel<LOG2L><<<count, sssp::kLargeNT, B::SMEM, st>>>(in, out, scale, work, tb, in_stride,
+                                                                               out_stride);
+  }
   return cudaGetLastError();
 }
 
@@ -273,22 +289,22 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
 }
 
 cudaError_t launch_dst(int log2L, const float2* in, float2* out, float scale, const TransformTables& tabs,
-                       cudaStream_t st, float2* work = nullptr, int bc = 0) {
+                       cudaStream_t st, float2* work = nullptr, int bc = 0, const sssp::StartArgs& sa = {}) {
   switch (log2L) {
     case 13: return launch_dst_large_t<13>(in, out, scale, work, tabs, st);
     case 14: return launch_dst_large_t<14>(in, out, scale, work, tabs, st);
     case 15: return launch_dst_large_t<15>(in, out, scale, work, tabs, st);
     case 16: return launch_dst_large_t<16>(in, out, scale, work, tabs, st);
-    case 3: return launch_dst_t<3>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 4: return launch_dst_t<4>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 5: return launch_dst_t<5>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 6: return launch_dst_t<6>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 7: return launch_dst_t<7>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 8: return launch_dst_t<8>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 9: return launch_dst_t<9>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 10: return launch_dst_t<10>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 11: return launch_dst_t<11>(in, out, scale, tabs, st, 1, 0, 0, bc);
-    case 12: return launch_dst_t<12>(in, out, scale, tabs, st, 1, 0, 0, bc);
+    case 3: return launch_dst_t<3>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 4: return launch_dst_t<4>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 5: return launch_dst_t<5>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 6: return launch_dst_t<6>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 7: return launch_dst_t<7>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 8: return launch_dst_t<8>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 9: return launch_dst_t<9>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 10: return launch_dst_t<10>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 11: return launch_dst_t<11>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
+    case 12: return launch_dst_t<12>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
   }
   return cudaErrorInvalidValue;
 }
@@ -717,24 +733,26 @@ pe_status pe_set_field(pe_plan* p, const float* u, int on_device, double r) {
   NvtxRange nvtx_("pe_set_field");
   if (!u) return fail(p, PE_ERR_ARG, "u is NULL");
   if (!std::isfinite(r)) return fail(p, PE_ERR_ARG, "r must be finite");
-  PE_CUDA(p, cudaMemcpyAsync(p->dStage, u, sizeof(float2) * p->N_user,
-                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, p->stream));
-  if (p->user_bc == PE_BC_NEUMANN) {
-    const int K = p->N / 2;
-    even_extend_kernel<<<(K + 255) / 256, 256, 0, p->stream>>>(p->dStage, K);
+  // a device field is read where it lies (complex values at an 8-byte boundary), others are staged
+  const float2* src = reinterpret_cast<const float2*>(u);
+  if (!on_device || reinterpret_cast<uintptr_t>(u) % sizeof(float2) != 0) {
+    PE_CUDA(p, cudaMemcpyAsync(p->dStage, u, sizeof(float2) * p->N_user,
+                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, p->stream));
+    src = p->dStage;
+  }
+  // one launch writes the spectral state, the field as given (Dirichlet: index 0 = boundary) and the
+  // cleared status word where the transform fits one CTA
+  sssp::StartArgs sa;
+  sa.field = p->dField;
+  sa.status = p->dStatus;
+  sa.mirror = p->user_bc == PE_BC_NEUMANN ? p->N / 2 : 0;
+  const bool fd = p->op == PE_OP_FD3, small = !fd && p->log2L <= kMaxSmemLog2;
+  if (!small) {  // FD-SSP marches depth values: index 0 the boundary, 1..N the field
+    sssp::sssp_start_kernel<sssp::kBcDirichlet><<<(p->L + 255) / 256, 256, 0, p->stream>>>(src, fd ? p->dYhat : nullptr,
+                                                                                            p->L, sa);
     PE_CUDA(p, cudaGetLastError());
   }
-  if (p->op == PE_OP_FD3) {  // FD-SSP marches depth values: index 0 the boundary, 1..N the field
-    PE_CUDA(p, cudaMemsetAsync(p->dYhat, 0, sizeof(float2), p->stream));
-    PE_CUDA(p, cudaMemcpyAsync(p->dYhat + 1, p->dStage, sizeof(float2) * p->N, cudaMemcpyDeviceToDevice, p->stream));
-  } else {
-    PE_CUDA(p, launch_dst(p->log2L, p->dStage, p->dYhat, 1.0f, p->tabs, p->stream, p->dWork, p->bc));
-  }
-  // the physical field as given (Dirichlet: index 0 = boundary)
-  if (p->off) PE_CUDA(p, cudaMemsetAsync(p->dField, 0, sizeof(float2), p->stream));
-  PE_CUDA(p, cudaMemcpyAsync(p->dField + p->off, p->dStage, sizeof(float2) * p->N, cudaMemcpyDeviceToDevice,
-                             p->stream));
-  PE_CUDA(p, cudaMemsetAsync(p->dStatus, 0, sizeof(int), p->stream));
+  if (!fd) PE_CUDA(p, launch_dst(p->log2L, src, p->dYhat, 1.0f, p->tabs, p->stream, p->dWork, p->bc, small ? sa : sssp::StartArgs{}));
   if (!on_device) PE_CUDA(p, cudaStreamSynchronize(p->stream));
   p->r_set = r;
   p->steps_done = 0;

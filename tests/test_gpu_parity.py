@@ -1417,3 +1417,52 @@ def test_parity_split_march_against_oracle(sssp, N, terms, absorb):
     for k in range(s.steps):  # the rows as magnitudes: every depth point, weighted by its own size
         got, want = 10.0 ** (-tl[k].astype(np.float64) / 20.0), 10.0 ** (-ref.tl[k] / 20.0)
         assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 12e-6 * math.log2(N + 1) / 8
+
+
+# ----------------------------------------------------------------------------- starters
+@pytest.mark.parametrize("N", [8191, 16383, 32767, 65535])
+def test_large_dst_tiles_equal_the_one_cta_kernel(sssp, N):
+    """The large transform with a CTA per tile (up to 32 fields) and with a CTA per field (beyond)
+    does the same arithmetic: the same bits, first and last field."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(N)
+    x = torch.randn(33, N, generator=g, dtype=torch.complex64, device="cuda")
+    pl = sssp.Plan(N, 100.0, 0.4, 5.0, 4)
+    many, few, one = torch.empty_like(x), torch.empty_like(x[:32]), torch.empty_like(x[:1])
+    pl.dst1_batch(x, many)
+    pl.dst1_batch(x[:32], few)
+    pl.dst1_batch(x[32:], one)
+    assert torch.equal(torch.view_as_real(many[:32]), torch.view_as_real(few))
+    assert torch.equal(torch.view_as_real(many[32:]), torch.view_as_real(one))
+    pl.close()
+
+
+@pytest.mark.parametrize("N,bc,op", [(7, "dirichlet", "spectral"), (255, "dirichlet", "fd3"), (1023, "dirichlet", "spectral"),
+                                     (64, "periodic", "spectral"), (9, "neumann", "spectral"), (1025, "neumann", "spectral"),
+                                     (8191, "dirichlet", "spectral")])
+def test_set_field_same_bits_from_host_device_and_odd_addresses(sssp, N, bc, op):
+    """A starter from host memory, from device memory and from a device address that is no multiple
+    of 8 bytes leaves the same state, the field as given, and a cleared status word."""
+    import torch
+    rng = np.random.default_rng(N)
+    u = (rng.standard_normal(N) + 1j * rng.standard_normal(N)).astype(np.complex64)
+    pl = sssp.Plan(N, 100.0, 0.4, 5.0, 4, bc=bc)
+    if op != "spectral":
+        pl.set_operator(op)
+        pl.set_profile(np.ones(N))
+    d = torch.from_numpy(u).cuda()
+    odd = torch.empty(2 * N + 1, dtype=torch.float32, device="cuda")
+    odd[1:] = torch.view_as_real(d).reshape(-1)
+    states = []
+    for where in ("host", "device", "odd"):
+        pl.inject_status(4)
+        if where == "host":
+            pl.set_field(u)
+        elif where == "device":
+            pl.set_field(d)
+        else:
+            pl._c(sssp.lib().pe_set_field(pl.handle, odd.data_ptr() + 4, 1, 0.0))
+        assert np.array_equal(pl.read_field(), u)  # no step marched: the carrier is 1
+        states.append(pl.save_state()[0])
+    assert np.array_equal(states[0], states[1]) and np.array_equal(states[0], states[2])
+    pl.close()
