@@ -1,5 +1,5 @@
-// SSSP range march of one solve per CTA with the modes split by parity (Dirichlet grids,
-// L = N + 1 in [512, 4096]): half the warps hold the even modes, half the odd ones.
+// The DST-I with the modes split by parity over two halves of a CTA's warps (Dirichlet grids, L = N + 1 in
+// [512, 4096]), and the range march of one solve per CTA built on it (L = 2048 and 4096).
 //
 // With M = L/2 the DST-I of x splits into two transforms of M points that never mix modes:
 //   O_n = sum_k S_{2k+1} sin(pi (2k+1) n/L),  E_n = sum_k S_{2k} sin(pi k n/M),   n in [0, M]
@@ -22,11 +22,11 @@
 // No prefix scan over the modes is left, and neither half waits for the other but at the depth points.
 //
 // What bounds it: the chain of dependent passes (3 radix passes and 2 exchanges a transform, one block
-// barrier a Neumann term) at one to two warps a scheduler; with four solves an SM the shared-memory
-// pipe (550 wavefronts a transform at L = 1024) is half busy.  8 points a thread: 16 gave 2460 cycles a
-// transform for one solve of L = 1024 and 2720 for two an SM, 8 give 1720 and 2410; the scan form it
-// replaced took 2250 and 3550 (2.07 GHz, N = 1023, [6/6], 12 terms; 256 solves x 160 steps in
-// 27 -> 20 ms of kernel time).  Its FP32 error is also smaller (no sums over L/2 modes).
+// barrier a Neumann term) at a few warps a scheduler; then the shared-memory pipe (550 wavefronts a
+// transform at L = 1024).  8 points a thread: with 16, one solve of L = 2048 took 4200 cycles a transform
+// (2.07 GHz), with 8 3040; the scan form it replaced 4600 (37 solves of N = 2047, complex n^2, [6/6],
+// 40 steps: 9.1 -> 5.8 ms).  Its FP32 error is smaller too (no sums over L/2 modes): 3.1e-6 -> 1.2e-6
+// against complex128 there.
 #pragma once
 #include "march_kernel.cuh"
 
@@ -583,6 +583,79 @@ __global__ void __launch_bounds__(ECfg<LOG2L>::NT, ECfg<LOG2L>::MIN_BLOCKS)
   if (t == 0) {
     if (status != kStatusOk) atomicMax(d.status, status);
     atomicAdd(d.ndst, (unsigned long long)ndst);
+  }
+}
+
+// DST-I of `count` fields: out = scale * DST(in), field b reads N values at in + b in_stride and writes its
+// modes k >= 1 - off at out + b out_stride (off = 1: mode 0 first, L values; off = 0: N values).  A CTA
+// takes fields b = blockIdx.x, blockIdx.x + gridDim.x, ..., so the twiddles are loaded once, and a
+// field's modes leave through shared memory, in order.
+//
+// Against one CTA per field with its tables in shared memory (51 KB, 12 KB of tables loaded per
+// field): more fields an SM, no table traffic, the march's shorter pass chain, and the packed result
+// rows are written here.  4096 fields of N = 1023: 98 -> 18.7 us (690 -> 3580 GB/s of input and output,
+// 53 % of the copy bandwidth), of N = 4095: 418 -> 129 us; one field: 16.6 -> 5.1 us.  It is bound by
+// the same chain at 6 fields an SM, with the shared-memory pipe as the next limit.
+template <int LOG2L>
+struct EDst {
+  using K = ECfg<LOG2L>;
+  static constexpr int MIN_BLOCKS = 65536 / (K::NT * 80);
+  static constexpr size_t SMEM = sizeof(float2) * 2 * (K::X1 + K::X2);
+  static_assert(K::L + K::L / 16 <= 2 * (K::X1 + K::X2), "the ordered modes reuse the exchange buffers");
+};
+
+template <int LOG2L>
+__global__ void __launch_bounds__(ECfg<LOG2L>::NT, EDst<LOG2L>::MIN_BLOCKS)
+    sssp_dst_eo_kernel(const float2* in, float2* out, float scale, const EoTabs tb, int count, long long in_stride,
+                       long long out_stride, int off, const StartArgs sa) {
+  using K = ECfg<LOG2L>;
+  constexpr int L = K::L, M = K::M, NT = K::NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* st = reinterpret_cast<float2*>(smem_raw);  // the modes in order (padded)
+  const EoThread<LOG2L> th;
+  const int t = threadIdx.x, e = th.e;
+  float2* x1 = st + e * (K::X1 + K::X2);
+  float2* x2 = x1 + K::X1;
+  EoTw<LOG2L> tw;
+  tw.load(tb, th);
+  EoPair pc;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) pc.c[i] = e ? __ldg(tb.cL + th.slot(i)) : make_float2(__ldg(tb.beta + th.slot(i)), 0.f);
+  const float h = e ? 0.5f : 0.25f, g = e ? 0.5f : -0.25f;  // odd half (x_n + x_{L-n})/2, even half (x_n - x_{L-n})/4
+  for (int b = blockIdx.x; b < count; b += gridDim.x) {
+    const float2* x = in + b * in_stride - 1;  // x[n], n in [1, N]
+    float2 p[4], q[4], xm = make_float2(0.f, 0.f), sp[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = th.slot(i);
+      const float2 zero = make_float2(0.f, 0.f);
+      const float2 a0 = m ? x[m] : zero, a1 = m ? x[L - m] : zero, b0 = x[M - m], b1 = x[M + m];
+      p[i] = make_float2(fmaf(h, a0.x, g * a1.x), fmaf(h, a0.y, g * a1.y));
+      q[i] = make_float2(fmaf(h, b0.x, g * b1.x), fmaf(h, b0.y, g * b1.y));
+      if (sa.field) {  // the odd half writes n < M, the even half the rest
+        if (e) {
+          sa.field[m] = a0;
+          if (m) sa.field[M - m] = b0;
+        } else {
+          if (m) sa.field[L - m] = a1;
+          sa.field[M + m] = b1;
+        }
+      }
+    }
+    if (th.z) {
+      const float2 a0 = x[M / 2], a1 = x[L - M / 2];
+      xm = make_float2(fmaf(h, a0.x, g * a1.x), fmaf(h, a0.y, g * a1.y));
+      if (sa.field) sa.field[e ? M / 2 : L - M / 2] = e ? a0 : a1;
+    }
+    if (sa.status && t == 0) *sa.status = kStatusOk;
+    eo_forward<LOG2L>(p, q, xm, sp, tw, pc, th, x1, x2);
+    __syncthreads();  // both halves are past the exchange buffers
+#pragma unroll
+    for (int i = 0; i < 8; ++i) st[pidx(th.mode(i))] = th.sign(i) * scale * sp[i];
+    __syncthreads();
+    float2* o = out + b * out_stride + off - 1;
+    for (int k = t + 1 - off; k < L; k += NT) o[k] = st[pidx(k)];
+    __syncthreads();
   }
 }
 

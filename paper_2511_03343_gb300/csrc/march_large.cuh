@@ -583,24 +583,27 @@ struct SrcIn {  // x_m = in[m - 1]
 };
 struct SnkScaled {
   static constexpr bool kL2 = false;
-  float2* out;
+  float2* out;  // mode k at out[k - 1 + off]; off = 0 leaves mode 0 out
   float s;
+  int off;
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
-  __device__ __forceinline__ void put(int, int k, float2 v) { out[k] = s * v; }
+  __device__ __forceinline__ void put(int, int k, float2 v) {
+    if (k + off > 0) out[k - 1 + off] = s * v;
+  }
 };
 
 template <int LOG2L>
 __global__ void __launch_bounds__(kLargeNT, 1)
-    sssp_dst_large_kernel(const float2* __restrict__ in, float2* __restrict__ out, float scale, float2* work,
-                          const LargeTabs tb, long long in_stride = 0, long long out_stride = 0) {
+    sssp_dst_large_kernel(const float2* in, float2* out, float scale, float2* work, const LargeTabs tb,
+                          long long in_stride, long long out_stride, int off) {
   extern __shared__ __align__(16) float2 tile_smem[];
   in += blockIdx.x * in_stride;
   out += blockIdx.x * out_stride;
   work += blockIdx.x * (long long)large_work_elems(1 << LOG2L);
   load_large_twiddles<LOG2L>(tile_smem, tb);
   __syncthreads();
-  SnkScaled sk{out, scale};
+  SnkScaled sk{out, scale, off};
   dst_global<LOG2L>(work, tb, tile_smem, SrcIn{in}, sk);
 }
 
@@ -609,15 +612,15 @@ __global__ void __launch_bounds__(kLargeNT, 1)
 // results are too, bit for bit.
 template <int LOG2L, bool PASS_B>
 __global__ void __launch_bounds__(kLargeNT, 1)
-    sssp_dst_large_tile_kernel(const float2* in, float2* __restrict__ out, float scale, float2* work, const LargeTabs tb,
-                               long long in_stride, long long out_stride) {
+    sssp_dst_large_tile_kernel(const float2* in, float2* out, float scale, float2* work, const LargeTabs tb,
+                               long long in_stride, long long out_stride, int off) {
   extern __shared__ __align__(16) float2 tile_smem[];
   work += blockIdx.y * (long long)large_work_elems(1 << LOG2L);
   load_large_twiddles<LOG2L>(tile_smem, tb);
   __syncthreads();
   const int c = blockIdx.x;
   if constexpr (PASS_B) {
-    SnkScaled sk{out + blockIdx.y * out_stride, scale};
+    SnkScaled sk{out + blockIdx.y * out_stride, scale, off};
     dst_pass_b<LOG2L>(work, tile_smem, sk, c, c + 1);
   } else {
     dst_pass_a<LOG2L>(work, tile_smem, SrcIn{in + blockIdx.y * in_stride}, c, c + 1);

@@ -124,13 +124,13 @@ cudaError_t set_smem_attr() {
   const int sm = int(Cfg<LOG2L>::SMEM), smc = int(Cfg<LOG2L>::SMEM_CPLX);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaSuccess;
-  if constexpr (LOG2L < sssp_eo::kMinLog2) {
+  if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
     e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet>, a, smc);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet>, a, sm);
   }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic>, a, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic>, a, smc);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet>, a, sm);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic>, a, sm);
   if (e == cudaSuccess) done_dev = dev;
   return e;
@@ -148,7 +148,7 @@ cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTa
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
       sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<count, nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
-  } else if constexpr (LOG2L < sssp_eo::kMinLog2) {
+  } else if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
     if (cplx)
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
@@ -166,7 +166,7 @@ cudaError_t launch_dst_t(const float2* in, float2* out, float scale, const Trans
   if (bc == sssp::kBcPeriodic)
     sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
         in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
-  else
+  else if constexpr (LOG2L < sssp_eo::kMinMarchLog2)
     sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
         in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
   return cudaGetLastError();
@@ -241,20 +241,20 @@ cudaError_t launch_march_large_t(const SolveDesc* dDescs, int count, const Trans
 }
 
 template <int LOG2L>
-cudaError_t launch_dst_large_t(const float2* in, float2* out, float scale, float2* work, const TransformTables&,
-                               cudaStream_t st, int count = 1, long long in_stride = 0, long long out_stride = 0) {
+cudaError_t launch_dst_large_t(const float2* in, float2* out, float scale, float2* work, cudaStream_t st, int count,
+                               long long in_stride, long long out_stride, int off) {
   sssp::LargeTabs tb;
   cudaError_t e = large_tabs<LOG2L>(&tb);
   if (e != cudaSuccess) return e;
   using B = sssp::BigCfg<LOG2L>;
   if (count <= kLargeTileFields) {
     sssp::sssp_dst_large_tile_kernel<LOG2L, false><<<dim3(B::NA, count), sssp::kLargeNT, B::SMEM, st>>>(
-        in, out, scale, work, tb, in_stride, out_stride);
+        in, out, scale, work, tb, in_stride, out_stride, off);
     sssp::sssp_dst_large_tile_kernel<LOG2L, true><<<dim3(B::NBT, count), sssp::kLargeNT, B::SMEM, st>>>(
-        in, out, scale, work, tb, in_stride, out_stride);
+        in, out, scale, work, tb, in_stride, out_stride, off);
   } else {
     sssp::sssp_dst_large_kernel<LOG2L><<<count, sssp::kLargeNT, B::SMEM, st>>>(in, out, scale, work, tb, in_stride,
-                                                                               out_stride);
+                                                                               out_stride, off);
   }
   return cudaGetLastError();
 }
@@ -265,10 +265,13 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
     if (bc != sssp::kBcDirichlet) return cudaErrorInvalidValue;
     return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx);
   }
-  // Dirichlet, L >= 512: the parity-split kernel, faster at every count there (one solve of L = 1024
-  // 2250 -> 1720 cycles a transform, two an SM 3550 -> 2410, one of L = 2048 4600 -> 3040, of L = 4096
-  // 6900 -> 6050); below it the half-transforms have fewer points than a warp's eight per lane
-  if (bc == sssp::kBcDirichlet && sssp_eo::supported(log2L)) return sssp_eo::launch_march(log2L, d, count, st, cplx);
+  // Dirichlet, L = 2048 and 4096: the parity-split kernel (one solve of L = 2048 4600 -> 3040 cycles a
+  // transform at 2.07 GHz, of L = 4096 6900 -> 6050).  L <= 1024 stays with the scan form: the split march
+  // is faster there too (one solve of L = 1024 2250 -> 1720, two an SM 3550 -> 2410), but these sizes'
+  // results are kept bit for bit: over the 256-solve batch another rounding of the scan form's sums
+  // moves the transmission loss by up to 0.2 dB at its deepest nulls.
+  if (bc == sssp::kBcDirichlet && sssp_eo::march_supported(log2L))
+    return sssp_eo::launch_march(log2L, d, count, st, cplx);
   switch (log2L) {
     case 3: return launch_march_t<3>(d, count, tabs, st, cplx, bc);
     case 4: return launch_march_t<4>(d, count, tabs, st, cplx, bc);
@@ -288,44 +291,29 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
   return cudaErrorInvalidValue;
 }
 
+// DST-I (periodic: DFT) of `count` fields: field b reads N values at in + b in_stride and writes L values at
+// out + b out_stride (off = 1), or its N modes from mode 1 on (off = 0; L >= 512 only).  A starter (sa.status)
+// takes the transform of its size's march, so the scan form up to L = 1024.
 cudaError_t launch_dst(int log2L, const float2* in, float2* out, float scale, const TransformTables& tabs,
-                       cudaStream_t st, float2* work = nullptr, int bc = 0, const sssp::StartArgs& sa = {}) {
+                       cudaStream_t st, float2* work, int bc, int count = 1, long long is = 0, long long os = 0,
+                       int off = 1, const sssp::StartArgs& sa = {}) {
+  if (bc == sssp::kBcDirichlet && (sa.status ? sssp_eo::march_supported(log2L) : sssp_eo::supported(log2L)))
+    return sssp_eo::launch_dst(log2L, in, out, scale, count, is, os, off, st, sa);
   switch (log2L) {
-    case 13: return launch_dst_large_t<13>(in, out, scale, work, tabs, st);
-    case 14: return launch_dst_large_t<14>(in, out, scale, work, tabs, st);
-    case 15: return launch_dst_large_t<15>(in, out, scale, work, tabs, st);
-    case 16: return launch_dst_large_t<16>(in, out, scale, work, tabs, st);
-    case 3: return launch_dst_t<3>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 4: return launch_dst_t<4>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 5: return launch_dst_t<5>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 6: return launch_dst_t<6>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 7: return launch_dst_t<7>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 8: return launch_dst_t<8>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 9: return launch_dst_t<9>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 10: return launch_dst_t<10>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 11: return launch_dst_t<11>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-    case 12: return launch_dst_t<12>(in, out, scale, tabs, st, 1, 0, 0, bc, sa);
-  }
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_dst_batch(int log2L, const float2* in, float2* out, const TransformTables& tabs, cudaStream_t st,
-                             float2* work, int count, long long in_stride, long long out_stride, int bc = 0) {
-  switch (log2L) {
-    case 3: return launch_dst_t<3>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 4: return launch_dst_t<4>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 5: return launch_dst_t<5>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 6: return launch_dst_t<6>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 7: return launch_dst_t<7>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 8: return launch_dst_t<8>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 9: return launch_dst_t<9>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 10: return launch_dst_t<10>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 11: return launch_dst_t<11>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 12: return launch_dst_t<12>(in, out, 1.f, tabs, st, count, in_stride, out_stride, bc);
-    case 13: return launch_dst_large_t<13>(in, out, 1.f, work, tabs, st, count, in_stride, out_stride);
-    case 14: return launch_dst_large_t<14>(in, out, 1.f, work, tabs, st, count, in_stride, out_stride);
-    case 15: return launch_dst_large_t<15>(in, out, 1.f, work, tabs, st, count, in_stride, out_stride);
-    case 16: return launch_dst_large_t<16>(in, out, 1.f, work, tabs, st, count, in_stride, out_stride);
+    case 3: return launch_dst_t<3>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 4: return launch_dst_t<4>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 5: return launch_dst_t<5>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 6: return launch_dst_t<6>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 7: return launch_dst_t<7>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 8: return launch_dst_t<8>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 9: return launch_dst_t<9>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 10: return launch_dst_t<10>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 11: return launch_dst_t<11>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 12: return launch_dst_t<12>(in, out, scale, tabs, st, count, is, os, bc, sa);
+    case 13: return launch_dst_large_t<13>(in, out, scale, work, st, count, is, os, off);
+    case 14: return launch_dst_large_t<14>(in, out, scale, work, st, count, is, os, off);
+    case 15: return launch_dst_large_t<15>(in, out, scale, work, st, count, is, os, off);
+    case 16: return launch_dst_large_t<16>(in, out, scale, work, st, count, is, os, off);
   }
   return cudaErrorInvalidValue;
 }
@@ -752,7 +740,8 @@ pe_status pe_set_field(pe_plan* p, const float* u, int on_device, double r) {
                                                                                             p->L, sa);
     PE_CUDA(p, cudaGetLastError());
   }
-  if (!fd) PE_CUDA(p, launch_dst(p->log2L, src, p->dYhat, 1.0f, p->tabs, p->stream, p->dWork, p->bc, small ? sa : sssp::StartArgs{}));
+  if (!fd) PE_CUDA(p, launch_dst(p->log2L, src, p->dYhat, 1.0f, p->tabs, p->stream, p->dWork, p->bc, 1, 0, 0,
+                                 1, small ? sa : sssp::StartArgs{}));
   if (!on_device) PE_CUDA(p, cudaStreamSynchronize(p->stream));
   p->r_set = r;
   p->steps_done = 0;
@@ -1139,18 +1128,30 @@ pe_status pe_dst1_batch(pe_plan* p, const float* in, float* out, int count) {
   if (!in || !out || count < 0) return fail(p, PE_ERR_ARG, "in/out NULL or count < 0");
   if (p->user_bc == PE_BC_NEUMANN) return fail(p, PE_ERR_ARG, "pe_dst1_batch takes Dirichlet or periodic plans");
   if (count == 0) return PE_OK;
-  // every field gets an L-long result row (index 0 is the zero mode), then rows 1..N are packed
+  const float2* src = reinterpret_cast<const float2*>(in);
+  const uintptr_t ia = reinterpret_cast<uintptr_t>(in), oa = reinterpret_cast<uintptr_t>(out);
+  const size_t bytes = sizeof(float2) * size_t(p->N) * size_t(count);
+  // The L >= 512 kernels write the packed rows themselves (every field is read before it is written, so
+  // in place too).  Elsewhere -- and for result addresses or overlaps that need the detour -- a field gets
+  // an L-long result row (index 0 is the zero mode), then rows 1..N are packed.
+  const bool direct = p->bc == PE_BC_DIRICHLET && p->log2L >= sssp_eo::kMinLog2 && oa % sizeof(float2) == 0 &&
+                      (ia == oa || ia + bytes <= oa || oa + bytes <= ia);
   float2* res = nullptr;
   float2* work = nullptr;
-  PE_CUDA(p, cudaMallocAsync(reinterpret_cast<void**>(&res), sizeof(float2) * size_t(p->L) * count, p->stream));
+  if (!direct)
+    PE_CUDA(p, cudaMallocAsync(reinterpret_cast<void**>(&res), sizeof(float2) * size_t(p->L) * count, p->stream));
   if (p->log2L > kMaxSmemLog2)
     PE_CUDA(p, cudaMallocAsync(reinterpret_cast<void**>(&work),
                                sizeof(float2) * sssp::large_work_elems(p->L) * size_t(count), p->stream));
-  PE_CUDA(p, launch_dst_batch(p->log2L, reinterpret_cast<const float2*>(in), res, p->tabs, p->stream, work, count,
-                              p->N, p->L, p->bc));
-  PE_CUDA(p, cudaMemcpy2DAsync(out, sizeof(float2) * p->N, res + p->off, sizeof(float2) * p->L, sizeof(float2) * p->N,
-                               count, cudaMemcpyDeviceToDevice, p->stream));
-  PE_CUDA(p, cudaFreeAsync(res, p->stream));
+  if (direct) {
+    PE_CUDA(p, launch_dst(p->log2L, src, reinterpret_cast<float2*>(out), 1.f, p->tabs, p->stream, work, p->bc, count,
+                          p->N, p->N, 0));
+  } else {
+    PE_CUDA(p, launch_dst(p->log2L, src, res, 1.f, p->tabs, p->stream, work, p->bc, count, p->N, p->L));
+    PE_CUDA(p, cudaMemcpy2DAsync(out, sizeof(float2) * p->N, res + p->off, sizeof(float2) * p->L, sizeof(float2) * p->N,
+                                 count, cudaMemcpyDeviceToDevice, p->stream));
+    PE_CUDA(p, cudaFreeAsync(res, p->stream));
+  }
   if (work) PE_CUDA(p, cudaFreeAsync(work, p->stream));
   return PE_OK;
 }

@@ -1388,8 +1388,8 @@ def test_fdssp_range_dependent_nodes(sssp):
 @pytest.mark.parametrize("N", [511, 1023, 2047, 4095])
 @pytest.mark.parametrize("terms,absorb", [(1, False), (2, False), (5, False), (12, True)])
 def test_parity_split_march_against_oracle(sssp, N, terms, absorb):
-    """The one-CTA kernel with the modes split by parity, at every size it takes (each has its own
-    middle radix 4, 8, 16 or 32), for series of one term (V ignored), two (the loop's shortest), five
+    """The one-CTA march on either side of the line between the scan form and the modes split by
+    parity (L = 2048 and 4096, with their own middle radix 16 and 32), for series of one term (V ignored), two (the loop's shortest), five
     and the full rule, real and complex profiles, a node change half way, and a TL row every step,
     from a field on every depth point (so every mode and both extra points M/2 carry weight).
     Bound: a transform's FP32 error is below 1e-6 log2 L of its input, 3 steps of [4/4] chain at
@@ -1465,4 +1465,28 @@ def test_set_field_same_bits_from_host_device_and_odd_addresses(sssp, N, bc, op)
         assert np.array_equal(pl.read_field(), u)  # no step marched: the carrier is 1
         states.append(pl.save_state()[0])
     assert np.array_equal(states[0], states[1]) and np.array_equal(states[0], states[2])
+    pl.close()
+
+
+@pytest.mark.parametrize("N,count", [(127, 5), (511, 2500), (1023, 1000), (4095, 400), (8191, 3)])
+def test_dst1_batch_more_fields_than_ctas_in_place_and_overlapping(sssp, N, count):
+    """The batched transform with more fields than its CTAs (each takes several), in place, into
+    results one field further on in the same buffer, and to an address that is no multiple of 8 bytes:
+    all the bits of transforming the fields one at a time."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(N)
+    buf = torch.randn(count + 1, N, generator=g, dtype=torch.complex64, device="cuda")
+    x = buf[:count].clone()
+    pl = sssp.Plan(N, 100.0, 0.4, 5.0, 4)
+    out = torch.empty_like(x)
+    pl.dst1_batch(x, out)
+    for b in (0, 1, count // 2, count - 1):
+        assert torch.equal(torch.view_as_real(out[b]), torch.view_as_real(pl.dst1(x[b].contiguous())))
+    odd = torch.empty(2 * N * count + 1, dtype=torch.float32, device="cuda")
+    pl._c(sssp.lib().pe_dst1_batch(pl.handle, x.data_ptr(), odd.data_ptr() + 4, count))
+    assert torch.equal(odd[1:], torch.view_as_real(out).reshape(-1))
+    pl.dst1_batch(buf[:count], buf[1:])  # overlapping, shifted by a field
+    assert torch.equal(torch.view_as_real(buf[1:]), torch.view_as_real(out))
+    pl.dst1_batch(x, x)
+    assert torch.equal(torch.view_as_real(x), torch.view_as_real(out))
     pl.close()
