@@ -50,7 +50,8 @@ struct SolveDesc {
   float2* field;         // L  physical envelope written at the end of the march
   float* tl;             // TL rows, N floats each
   int* status;           // device status word
-  unsigned long long* ndst;  // number of DST-I transforms executed (accumulated)
+  unsigned long long* ndst;  // number of DST-I transforms executed (accumulated); the next word counts the
+                             // finished CTAs of a march whose TL rows are split over CTAs (0 between marches)
   float2 beta[kMaxStages];   // (L/2)(1 - a_j/b_j)
   double r0;             // range at the start of this march
   double dr;
@@ -656,6 +657,9 @@ __device__ __forceinline__ void record_tl(Smem<LOG2L, PPT>& sm, const SolveDesc&
 
 // ---------------------------------------------------------------------------------------
 // The persistent march: blockIdx.x selects the solve; thread t owns the modes [P t, P t + P).
+// A solve without V (terms <= 1) only transforms for its TL rows, and those do not depend on one another:
+// gridDim.y CTAs all take the (cheap, diagonal) steps, each transforms every gridDim.y-th row, and the last
+// to finish writes the state.  100 steps of N = 255 with a row each: 208 us on one CTA, see launch_march.
 // ---------------------------------------------------------------------------------------
 template <int LOG2L, bool CPLX, int BC, int PPT = 8>
 __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOCKS)
@@ -675,6 +679,7 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
   }
   load_tables<LOG2L, PPT>(sm.tw, sm.sinw, tw_g, sin_g);
   __syncthreads();
+  if (d.terms > 1 && blockIdx.y > 0) return;
   TwRegs<LOG2L, P> twr_v;
   const TwRegs<LOG2L, P>* twr = nullptr;
   if constexpr (C::TWREG) {
@@ -731,10 +736,23 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
       for (int i = 0; i < P; ++i) y[i] = ffmul(G[i], y[i]);
       const long long gs = d.step0 + s + 1;
       if (d.tl_every > 0 && gs % d.tl_every == 0) {
-        record_tl<LOG2L, BC, P>(sm, d, y, out_scale, s, nrec);
-        ++ndst;
+        if (nrec % int(gridDim.y) == int(blockIdx.y)) {
+          record_tl<LOG2L, BC, P>(sm, d, y, out_scale, s, nrec);
+          ++ndst;
+        }
         ++nrec;
       }
+    }
+    if (gridDim.y > 1) {  // every CTA has read the state it started from: the last one writes the new state
+      __shared__ bool last;
+      __syncthreads();
+      if (t == 0) {
+        __threadfence();
+        last = atomicInc(reinterpret_cast<unsigned*>(d.ndst + 1), gridDim.y - 1) == gridDim.y - 1;
+        if (!last) atomicAdd(d.ndst, (unsigned long long)ndst);
+      }
+      __syncthreads();
+      if (!last) return;
     }
   } else {
     for (int s = 0; s < d.steps && status == kStatusOk; ++s) {

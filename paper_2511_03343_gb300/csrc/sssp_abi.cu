@@ -138,21 +138,21 @@ cudaError_t set_smem_attr() {
 
 template <int LOG2L>
 cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTables& tabs, cudaStream_t st,
-                           bool cplx, int bc) {
+                           bool cplx, int bc, int split) {
   cudaError_t e = set_smem_attr<LOG2L>();
   if (e != cudaSuccess) return e;
   const int nt = Cfg<LOG2L>::NT;
   const size_t sm = Cfg<LOG2L>::SMEM, smc = Cfg<LOG2L>::SMEM_CPLX;
   if (bc == sssp::kBcPeriodic) {
     if (cplx)
-      sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
+      sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<dim3(count, split), nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
-      sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<count, nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
+      sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<dim3(count, split), nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
   } else if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
     if (cplx)
-      sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet><<<count, nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
+      sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet><<<dim3(count, split), nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
-      sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet><<<count, nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
+      sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet><<<dim3(count, split), nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
   }
   return cudaGetLastError();
 }
@@ -259,11 +259,17 @@ cudaError_t launch_dst_large_t(const float2* in, float2* out, float scale, float
   return cudaGetLastError();
 }
 
+// `iso_rows`: the most TL rows of a solve of the group that takes no Neumann terms (0: none).  The scan-form
+// kernel splits such rows over CTAs while the device has room for them: one solve of N = 255, 100 steps
+// with a row each 208 us on one CTA,
+// 48 us on 100 (march call to completion).
 cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const TransformTables& tabs, cudaStream_t st,
-                         bool cplx, int bc, int ppt = 8) {
+                         bool cplx, int bc, int ppt, int iso_rows) {
+  constexpr int kRoom = 304;  // two CTAs on each of the 152 SMs
+  const int split = std::max(1, std::min(iso_rows, kRoom / count));
   if (ppt != 8) {  // the one-CTA kernel at 4 or 16 points per thread (Dirichlet, L <= 4096)
     if (bc != sssp::kBcDirichlet) return cudaErrorInvalidValue;
-    return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx);
+    return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx, split);
   }
   // Dirichlet, L = 2048 and 4096: the parity-split kernel (one solve of L = 2048 4600 -> 3040 cycles a
   // transform at 2.07 GHz, of L = 4096 6900 -> 6050).  L <= 1024 stays with the scan form: the split march
@@ -273,16 +279,16 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
   if (bc == sssp::kBcDirichlet && sssp_eo::march_supported(log2L))
     return sssp_eo::launch_march(log2L, d, count, st, cplx);
   switch (log2L) {
-    case 3: return launch_march_t<3>(d, count, tabs, st, cplx, bc);
-    case 4: return launch_march_t<4>(d, count, tabs, st, cplx, bc);
-    case 5: return launch_march_t<5>(d, count, tabs, st, cplx, bc);
-    case 6: return launch_march_t<6>(d, count, tabs, st, cplx, bc);
-    case 7: return launch_march_t<7>(d, count, tabs, st, cplx, bc);
-    case 8: return launch_march_t<8>(d, count, tabs, st, cplx, bc);
-    case 9: return launch_march_t<9>(d, count, tabs, st, cplx, bc);
-    case 10: return launch_march_t<10>(d, count, tabs, st, cplx, bc);
-    case 11: return launch_march_t<11>(d, count, tabs, st, cplx, bc);
-    case 12: return launch_march_t<12>(d, count, tabs, st, cplx, bc);
+    case 3: return launch_march_t<3>(d, count, tabs, st, cplx, bc, split);
+    case 4: return launch_march_t<4>(d, count, tabs, st, cplx, bc, split);
+    case 5: return launch_march_t<5>(d, count, tabs, st, cplx, bc, split);
+    case 6: return launch_march_t<6>(d, count, tabs, st, cplx, bc, split);
+    case 7: return launch_march_t<7>(d, count, tabs, st, cplx, bc, split);
+    case 8: return launch_march_t<8>(d, count, tabs, st, cplx, bc, split);
+    case 9: return launch_march_t<9>(d, count, tabs, st, cplx, bc, split);
+    case 10: return launch_march_t<10>(d, count, tabs, st, cplx, bc, split);
+    case 11: return launch_march_t<11>(d, count, tabs, st, cplx, bc, split);
+    case 12: return launch_march_t<12>(d, count, tabs, st, cplx, bc, split);
     case 13: return launch_march_large_t<13>(d, count, tabs, st);
     case 14: return launch_march_large_t<14>(d, count, tabs, st);
     case 15: return launch_march_large_t<15>(d, count, tabs, st);
@@ -447,6 +453,11 @@ cudaError_t tables_for(const pe_plan* p, int ppt, TransformTables* out) {
   return get_tables(p->device, p->log2L, out, ppt);
 }
 
+// TL rows of a march that takes no Neumann terms (the isovelocity step), else 0
+int iso_rows(const SolveDesc& d) {
+  return d.terms <= 1 ? int(std::min<long long>(records_between(d.step0, d.step0 + d.steps, d.tl_every), 1 << 20)) : 0;
+}
+
 // Fill the descriptor for one march of `steps` steps and reserve its TL rows.
 pe_status prepare_desc(pe_plan* p, int steps, SolveDesc* d) {
   if (!p->field_set) return fail(p, PE_ERR_STATE, "pe_march before pe_set_field");
@@ -491,6 +502,12 @@ pe_status prepare_desc(pe_plan* p, int steps, SolveDesc* d) {
   p->tl_rows += recs;
   p->steps_done += steps;
   return PE_OK;
+}
+
+int group_iso_rows(const std::vector<SolveDesc>& g) {
+  int rows = 0;
+  for (const SolveDesc& d : g) rows = std::max(rows, iso_rows(d));
+  return rows;
 }
 
 pe_status check_status(pe_plan* p) {
@@ -692,7 +709,7 @@ pe_status pe_plan_create_bc(pe_plan** out, int N, double H, double k0, double dr
   if (log2L > kMaxSmemLog2 &&
       (e = cudaMalloc(&p->dWork, sizeof(float2) * sssp::large_work_elems(L))) != cudaSuccess)
     return bail(e, "cudaMalloc(workspace)");
-  if ((e = cudaMalloc(&p->dNdst, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = cudaMalloc(&p->dNdst, 2 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = cudaMalloc(&p->dDesc, sizeof(SolveDesc))) != cudaSuccess) return bail(e, "cudaMalloc");
   p->desc_cap = sizeof(SolveDesc);
   if ((e = cudaMemcpy(p->dR, R.data(), sizeof(float4) * R.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
@@ -700,7 +717,7 @@ pe_status pe_plan_create_bc(pe_plan** out, int N, double H, double k0, double dr
   if ((e = cudaMemcpy(p->dB, B.data(), sizeof(float2) * B.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
   if ((e = cudaMemcpy(p->dG, G.data(), sizeof(float4) * L, cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
   if ((e = cudaMemset(p->dStatus, 0, sizeof(int))) != cudaSuccess) return bail(e, "memset");
-  if ((e = cudaMemset(p->dNdst, 0, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "memset");
+  if ((e = cudaMemset(p->dNdst, 0, 2 * sizeof(unsigned long long))) != cudaSuccess) return bail(e, "memset");
   if ((e = cudaMemset(p->dYhat, 0, sizeof(float2) * L)) != cudaSuccess) return bail(e, "memset");
   if ((e = cudaMemset(p->dField, 0, sizeof(float2) * L)) != cudaSuccess) return bail(e, "memset");
   *out = p;
@@ -869,7 +886,7 @@ pe_status pe_march(pe_plan* p, int steps) {
     const int ppt = (p->log2L <= kMaxSmemLog2) ? shape_of(p) : 8;
     TransformTables tb;
     PE_CUDA(p, tables_for(p, ppt, &tb));
-    PE_CUDA(p, launch_march(p->log2L, p->dDesc, 1, tb, p->stream, cplx, p->bc, ppt));
+    PE_CUDA(p, launch_march(p->log2L, p->dDesc, 1, tb, p->stream, cplx, p->bc, ppt, iso_rows(d)));
   }
   return PE_OK;
 }
@@ -993,7 +1010,7 @@ pe_status pe_march_batch_steps(pe_plan** plans, const int* steps, int count) {
                                              std::get<4>(kv.first) & 1));
     else
       PE_CUDA(p0, launch_march(std::get<0>(kv.first), p0->dDesc, int(kv.second.size()), tabs[kv.first], p0->stream,
-                               std::get<1>(kv.first), std::get<2>(kv.first), std::get<4>(kv.first)));
+                               std::get<1>(kv.first), std::get<2>(kv.first), std::get<4>(kv.first), group_iso_rows(kv.second)));
     return PE_OK;
   }
   // several groups (grid sizes / kernels): each on its own stream, forked from the plan's stream
@@ -1025,7 +1042,7 @@ pe_status pe_march_batch_steps(pe_plan** plans, const int* steps, int count) {
                                              std::get<4>(kv.first) & 1));
     else
       PE_CUDA(p0, launch_march(std::get<0>(kv.first), dd, int(kv.second.size()), tabs[kv.first], st,
-                               std::get<1>(kv.first), std::get<2>(kv.first), std::get<4>(kv.first)));
+                               std::get<1>(kv.first), std::get<2>(kv.first), std::get<4>(kv.first), group_iso_rows(kv.second)));
     PE_CUDA(p0, cudaEventRecord(bl->done[g], st));
     PE_CUDA(p0, cudaStreamWaitEvent(p0->stream, bl->done[g], 0));
     ++g;

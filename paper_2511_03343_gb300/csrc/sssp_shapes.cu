@@ -15,7 +15,8 @@ namespace sssp_shapes {
 namespace {
 
 template <int LOG2L, int PPT, bool CPLX>
-cudaError_t launch_t(const sssp::SolveDesc* d, int count, const float2* tw, const float* sinw, cudaStream_t st) {
+cudaError_t launch_t(const sssp::SolveDesc* d, int count, const float2* tw, const float* sinw, cudaStream_t st,
+                     int split) {
   using C = sssp::Cfg<LOG2L, PPT>;
   const size_t sm = CPLX ? C::SMEM_CPLX : C::SMEM;
   static std::mutex mu;
@@ -32,25 +33,26 @@ cudaError_t launch_t(const sssp::SolveDesc* d, int count, const float2* tw, cons
       done.insert(dev);
     }
   }
-  sssp::sssp_march_kernel<LOG2L, CPLX, sssp::kBcDirichlet, PPT><<<count, C::NT, sm, st>>>(d, tw, sinw);
+  sssp::sssp_march_kernel<LOG2L, CPLX, sssp::kBcDirichlet, PPT><<<dim3(count, split), C::NT, sm, st>>>(d, tw, sinw);
   return cudaGetLastError();
 }
 
 template <int LOG2L, int PPT>
 cudaError_t launch_c(const sssp::SolveDesc* d, int count, const float2* tw, const float* sinw, cudaStream_t st,
-                     bool cplx) {
-  return cplx ? launch_t<LOG2L, PPT, true>(d, count, tw, sinw, st) : launch_t<LOG2L, PPT, false>(d, count, tw, sinw, st);
+                     bool cplx, int split) {
+  return cplx ? launch_t<LOG2L, PPT, true>(d, count, tw, sinw, st, split)
+              : launch_t<LOG2L, PPT, false>(d, count, tw, sinw, st, split);
 }
 
 template <int PPT>
 cudaError_t launch_p(int log2L, const sssp::SolveDesc* d, int count, const float2* tw, const float* sinw,
-                     cudaStream_t st, bool cplx) {
+                     cudaStream_t st, bool cplx, int split) {
   switch (log2L) {
-    case 8: return launch_c<8, PPT>(d, count, tw, sinw, st, cplx);
-    case 9: return launch_c<9, PPT>(d, count, tw, sinw, st, cplx);
-    case 10: return launch_c<10, PPT>(d, count, tw, sinw, st, cplx);
-    case 11: return launch_c<11, PPT>(d, count, tw, sinw, st, cplx);
-    case 12: return launch_c<12, PPT>(d, count, tw, sinw, st, cplx);
+    case 8: return launch_c<8, PPT>(d, count, tw, sinw, st, cplx, split);
+    case 9: return launch_c<9, PPT>(d, count, tw, sinw, st, cplx, split);
+    case 10: return launch_c<10, PPT>(d, count, tw, sinw, st, cplx, split);
+    case 11: return launch_c<11, PPT>(d, count, tw, sinw, st, cplx, split);
+    case 12: return launch_c<12, PPT>(d, count, tw, sinw, st, cplx, split);
   }
   return cudaErrorInvalidValue;
 }
@@ -82,9 +84,10 @@ size_t smem_bytes(int log2L, int ppt, bool cplx) {
 }
 
 cudaError_t launch_march(int log2L, int ppt, const sssp::SolveDesc* d, int count, const float2* tw,
-                         const float* sinw, cudaStream_t st, bool cplx) {
+                         const float* sinw, cudaStream_t st, bool cplx, int split) {
   if (!supported(log2L, ppt)) return cudaErrorInvalidValue;
-  return ppt == 4 ? launch_p<4>(log2L, d, count, tw, sinw, st, cplx) : launch_p<16>(log2L, d, count, tw, sinw, st, cplx);
+  return ppt == 4 ? launch_p<4>(log2L, d, count, tw, sinw, st, cplx, split)
+                  : launch_p<16>(log2L, d, count, tw, sinw, st, cplx, split);
 }
 
 }  // namespace sssp_shapes

@@ -1490,3 +1490,45 @@ def test_dst1_batch_more_fields_than_ctas_in_place_and_overlapping(sssp, N, coun
     pl.dst1_batch(x, x)
     assert torch.equal(torch.view_as_real(x), torch.view_as_real(out))
     pl.close()
+
+
+# ----------------------------------------------------------------------------- isovelocity rows over CTAs
+@pytest.mark.parametrize("N,bc,shape,count,steps,tl_every", [
+    (7, "dirichlet", 8, 1, 9, 1), (255, "dirichlet", 8, 1, 400, 1), (255, "dirichlet", 4, 1, 25, 2),
+    (255, "dirichlet", 16, 1, 25, 2), (1023, "dirichlet", 8, 100, 13, 3), (64, "periodic", 8, 2, 17, 1),
+    (65, "neumann", 8, 1, 17, 4), (255, "dirichlet", 8, 305, 6, 1)])
+def test_isovelocity_rows_split_over_ctas(sssp, N, bc, shape, count, steps, tl_every):
+    """A march without Neumann terms shares its TL rows between CTAs (more rows than CTAs, fewer, one CTA a
+    solve for large batches, a solve with Neumann terms in the same launch): the bits, the transform count
+    and the resumed march are those of marching one step at a time, where a march has at most one row."""
+    solves = []
+    for i in range(count):
+        s = inputs.isovelocity(N=N, freq=100.0 + 0.1 * i, steps=steps, bc=bc)
+        n = np.arange(1, N + 1)
+        s.u0 = np.sin(0.7 * n * (1 + i % 3)) + 1j * np.cos(0.3 * n)
+        solves.append(s)
+    if bc == "dirichlet":
+        solves.append(inputs.munk(N=N, freq=0.1 * (N + 1), dr=100.0, pade_order=4, steps=steps))
+
+    def plans():
+        ps = [sssp.plan_for(s, tl_every=tl_every) for s in solves]
+        for p in ps:
+            p.set_shape(shape)
+        return ps
+
+    a, b = plans(), plans()
+    for _ in range(2):  # the second march resumes from the state the first one's last CTA wrote
+        if len(a) == 1:
+            a[0].march(steps)
+        else:
+            sssp.march_batch(a, steps)
+        for _ in range(steps):
+            sssp.march_batch(b, 1)
+    for k in sorted({0, len(a) // 2, len(a) - 1}):
+        assert np.array_equal(a[k].read_field(), b[k].read_field())
+        ta, tb = a[k].read_tl(), b[k].read_tl()
+        assert ta[0].shape[0] == 2 * steps // tl_every and np.array_equal(ta[0], tb[0]) and np.array_equal(ta[1], tb[1])
+        if solves[k].neumann_terms <= 1:
+            assert a[k].transform_count() == 2 * steps // tl_every + 2
+    for p in a + b:
+        p.close()
