@@ -229,8 +229,9 @@ pe_status pe_dst1_noalloc(const float* in, float* out, int N, void* cuda_stream)
 
 /*
  * Which kernel marches a plan (no counterpart in the paper, which gives no implementation).
- *   PE_KERNEL_CTA      one CTA per solve, the field in that SM's shared memory (N + 1 <= 4096) or
- *                      in a per-plan global workspace (larger grids);
+ *   PE_KERNEL_CTA      one CTA per solve, the field in that SM's shared memory (N + 1 <= 4096); larger
+ *                      grids in a per-plan global workspace, by one CTA in large batches, else by 2 or 4
+ *                      that share the transforms' tiles (the same bits either way);
  *   PE_KERNEL_CLUSTER  one solve over a thread-block cluster of 8 or 16 CTAs (the cluster shape below),
  *                      every length-(N + 1) array in the cluster's distributed shared memory and
  *                      each DST-I of Section 3.1 as local FFTs plus one all-to-all exchange;

@@ -1,14 +1,17 @@
 // SSSP range march for grids larger than one CTA's shared memory (L = N + 1 = 8192 .. 65536).
 //
+// A solve is marched by a cluster of 1, 2 or 4 CTAs that share its tiles.
 // Same method as march_kernel.cuh (product-form Pade stages with hi/lo multipliers, Neumann
 // series, spectral-resident field), but every length-L array lives in a per-solve workspace
-// in global memory (L2-resident for a single solve, HBM for large batches), one CTA of 512
-// threads per solve, with a __syncthreads between passes (global writes are visible to the
-// block after it).  The DST-I here is the DFT of the odd extension in two passes of
+// in global memory (L2-resident for a few solves, HBM for large batches).  CTAs of 512 threads, one per
+// solve in large batches, else a cluster of 2 or 4 that shares the solve's tiles, with a barrier
+// between passes (global writes are visible to the CTAs after it).  The DST-I here is the DFT of the odd extension in two passes of
 // shared-memory tiles (see dst_global), with no prefix scan: the scan form's odd outputs lose
 // accuracy like sqrt(L) (3.6e-5 relative at L = 65536 in FP32), which these grids cannot afford.
 // Element-wise work walks the natural index i = t + 512 q, so every access is coalesced.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "march_kernel.cuh"
 
 namespace sssp {
@@ -30,22 +33,6 @@ struct CfgL {
   static constexpr int NW = NT / 32;
   static constexpr int PER = L / NT;        // elements per thread in element-wise loops
 };
-
-// block sum of one float; every thread gets the same total (red: NW floats of shared memory)
-template <int LOG2L>
-__device__ __forceinline__ float block_sum(float v, float* red) {
-  using C = CfgL<LOG2L>;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();  // previous users of red are done
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float s = (lane < C::NW) ? red[lane] : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
 
 // A hint that moves the 128-byte line holding p into the L2 (no registers held; p is always an
 // element of the arrays the pass reads).  Operands are fetched this way a tile before their
@@ -94,6 +81,10 @@ struct BigCfg {
   static constexpr int R = 1 << LOG2R, NT1 = L / R;
   // two tile buffers, the P- and Q-point twiddle tables, then the three tables above (all hi + lo)
   static constexpr size_t SMEM = sizeof(float2) * 2 * size_t(BUF) + sizeof(float4) * (P + Q + R + NT1 + Q / 2);
+  // the march also holds the two buffers of a one-warp FFT (the column Q/2 or the row P/2)
+  static constexpr size_t SMEM_MARCH = SMEM + sizeof(float2) * 2 * (RSP > RSQ ? RSP : RSQ);
+  static constexpr int CTAS = NA - 1;  // CTAs of a march's cluster: a tile of each pass each
+  static_assert(NA == NBT, "as many tiles in either pass");
 };
 
 // Tile FFTs use radix-16 Stockham passes (radix min(16, F/NS) at span NS), one butterfly of 16
@@ -212,6 +203,7 @@ __device__ __forceinline__ void dst_pass_a(float2* W, float2* sm, const SRC& src
   };
   if (c0 + 1 < c1) l2A(c0 + 1);
   loadA(c0);
+#pragma unroll 1
   for (int c = c0; c < c1; ++c) {
     const int cb = c < NA - 1 ? c * TC : QH - TC + 1;
 #pragma unroll
@@ -301,6 +293,7 @@ __device__ __forceinline__ void dst_pass_b(const float2* W, float2* sm, SNK& snk
     return true;
   };
   loadB(t0);
+#pragma unroll 1
   for (int tile = t0; tile < t1; ++tile) {
 #pragma unroll
     for (int q = 0; q < PH; ++q) {
@@ -351,6 +344,7 @@ __device__ __forceinline__ void dst_pass_b(const float2* W, float2* sm, SNK& snk
         }
       }
     }
+    snk.tile_end(tile - t0);
     __syncthreads();
   }
 }
@@ -364,6 +358,123 @@ template <int LOG2L, class SRC, class SNK>
 __device__ void dst_global(float2* W, const LargeTabs& tb, float2* sm, const SRC& src, SNK& snk) {
   dst_pass_a<LOG2L>(W, sm, src, 0, BigCfg<LOG2L>::NA);
   dst_pass_b<LOG2L>(W, sm, snk, 0, BigCfg<LOG2L>::NBT);
+}
+
+// One FFT of 2^LOG2F points by one warp (the same passes as a tile's); returns the buffer with the result
+template <int LOG2F, int NS>
+__device__ __forceinline__ float2* wfft(float2* src, float2* dst, const float4* tw) {
+  constexpr int F = 1 << LOG2F;
+  if constexpr (NS >= F) {
+    return src;
+  } else {
+    constexpr int RAD = large_rad(F, NS), NB = F / RAD, OFF = large_twoff(F, NS);
+#pragma unroll 1
+    for (int jj = threadIdx.x & 31; jj < NB; jj += 32) {
+      float2 v[RAD];
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) v[r] = src[pidx(jj + r * NB)];
+      const int k = jj & (NS - 1);
+      if constexpr (NS > 1) {
+#pragma unroll
+        for (int r = 1; r < RAD; ++r) v[r] = ffmul(tw[OFF + (r - 1) * NS + k], v[r]);
+      }
+      dftR<RAD>(v);
+#pragma unroll
+      for (int r = 0; r < RAD; ++r) dst[pidx((jj - k) * RAD + k + r * NS)] = v[r];
+    }
+    __syncwarp();
+    return wfft<LOG2F, NS * RAD>(dst, src, tw);
+  }
+}
+
+// pass A of the column Q/2 alone, by one warp (the tiles [0, NA - 1) hold the columns before it)
+template <int LOG2L, class SRC>
+__device__ __forceinline__ void dst_last_col(float2* W, float2* sm, const SRC& src) {
+  using C = BigCfg<LOG2L>;
+  constexpr int L = C::L, P = C::P, Q = C::Q, QH = Q / 2, QS = QH + 1;
+  const float4* twP = reinterpret_cast<const float4*>(sm + 2 * C::BUF);
+  const float4* tlo = twP + P + Q;
+  const float4* thi = tlo + C::R;
+  float2* b0 = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(sm) + C::SMEM);
+  float2* b1 = b0 + (C::RSP > C::RSQ ? C::RSP : C::RSQ);
+  const int lane = threadIdx.x & 31;
+  float2 z[P / 32];
+#pragma unroll
+  for (int q = 0; q < P / 32; ++q) {
+    const int n = Q * (lane + 32 * q) + QH;
+    const float2 x = n < L ? src(n, true) : src(2 * L - n, false);
+    z[q] = n < L ? x : make_float2(-x.x, -x.y);
+  }
+#pragma unroll
+  for (int q = 0; q < P / 32; ++q) b0[pidx(lane + 32 * q)] = z[q];
+  __syncwarp();
+  const float2* F = wfft<C::LOG2P, 1>(b0, b1, twP);
+  for (int k1 = lane; k1 < P; k1 += 32) {
+    const int e = QH * k1;
+    W[k1 * QS + QH] = ffmul(thi[e >> C::LOG2R], ffmul(tlo[e & (C::R - 1)], F[pidx(k1)]));
+  }
+  __syncwarp();
+}
+
+// pass B of the row P/2 alone, by one warp (its own partner: only the outputs k2 < Q/2 are kept)
+template <int LOG2L, class SNK>
+__device__ __forceinline__ void dst_last_row(const float2* W, float2* sm, SNK& snk) {
+  using C = BigCfg<LOG2L>;
+  constexpr int P = C::P, Q = C::Q, QH = Q / 2, QS = QH + 1;
+  const float4* twQ = reinterpret_cast<const float4*>(sm + 2 * C::BUF) + P;
+  const float4* tq = twQ + Q + C::R + C::NT1;
+  float2* b0 = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(sm) + C::SMEM);
+  float2* b1 = b0 + (C::RSP > C::RSQ ? C::RSP : C::RSQ);
+  const int lane = threadIdx.x & 31;
+  const float2* row = W + (P / 2) * QS;
+  for (int n = lane; n <= QH; n += 32) {
+    const float2 v = row[n];
+    b0[pidx(n)] = v;
+    if (n > 0 && n < QH) {
+      const float4 w = tq[n];
+      b0[pidx(Q - n)] = ffmul(make_float4(w.x, -w.y, w.z, -w.w), make_float2(-v.x, -v.y));
+    }
+  }
+  __syncwarp();
+  const float2* F = wfft<C::LOG2Q, 1>(b0, b1, twQ);
+  // lane i < G takes the outputs i + G q, as warp i does in the last tile of a one-CTA pass
+  constexpr int G = kLargeNT / C::TR;
+  if (lane < G) {
+    for (int k2 = lane; k2 < QH; k2 += G) {
+      const int k = P / 2 + P * k2;
+      const float2 zk = F[pidx(k2)];
+      snk.prefetch(0, k);
+      snk.put(0, k, make_float2(-0.5f * zk.y, 0.5f * zk.x));
+    }
+  }
+  snk.row_end(C::CTAS, lane);
+  __syncwarp();
+}
+
+// Barrier over the CTAs of a solve, ordering their global memory accesses too
+template <int NC>
+__device__ __forceinline__ void solve_sync() {
+  if constexpr (NC == 1) __syncthreads();
+  else cooperative_groups::this_cluster().sync();
+}
+
+// The transform by the NC CTAs of a solve (rank: this one): each takes its share of the tiles of either
+// pass, the last warp of the last CTA the odd column and row (one CTA: a last, overlapping tile does).
+// The barrier between the passes orders the intermediate; the caller's barrier after it the results.
+template <int LOG2L, int NC, class SRC, class SNK>
+__device__ void dst_cluster(float2* W, float2* sm, const SRC& src, SNK& snk, int rank) {
+  if constexpr (NC == 1) {
+    dst_pass_a<LOG2L>(W, sm, src, 0, BigCfg<LOG2L>::NA);
+    dst_pass_b<LOG2L>(W, sm, snk, 0, BigCfg<LOG2L>::NBT);
+  } else {
+    constexpr int T = BigCfg<LOG2L>::CTAS / NC;
+    const bool odd = rank == NC - 1 && int(threadIdx.x) >= kLargeNT - 32;
+    if (odd) dst_last_col<LOG2L>(W, sm, src);
+    dst_pass_a<LOG2L>(W, sm, src, rank * T, (rank + 1) * T);
+    solve_sync<NC>();
+    if (odd) dst_last_row<LOG2L>(W, sm, snk);
+    dst_pass_b<LOG2L>(W, sm, snk, rank * T, (rank + 1) * T);
+  }
 }
 
 // sources (depth or spectral values the transform reads) and sinks (where its outputs go)
@@ -411,12 +522,15 @@ struct SrcScaled {  // x_m = s y_m
   __device__ __forceinline__ void l2(int m) const { l2_prefetch(y + m); }
 };
 // A sink takes put(q, k, S_k) for its q-th output of a tile; prefetch(q, k) is called for the
-// same (q, k) before the tile's FFT, so a sink can load its own operands early.
+// same (q, k) before the tile's FFT, so a sink can load its own operands early; tile_end(i) after the
+// thread's last output of the i-th tile of its CTA, row_end(CTAS, lane) after the odd row of a cluster's march.
 struct SnkArr {
   static constexpr bool kL2 = false;  // write-only: no operands to fetch
   float2* a;
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
+  __device__ __forceinline__ void tile_end(int) {}
+  __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) { a[k] = v; }
 };
 // The partial sum w_j = t_0 + t_1 + .. is kept itself (not t_1 + .. beside t_0), so a term
@@ -430,8 +544,22 @@ struct SnkTerm {  // t_m = B_k S_k: w += t_m, X = t_m, and the norm partials of 
   const float2* B;
   float2* w;
   float2* X;
+  float2* red;  // shared memory: the norm partials of tile i and warp v at i NW + v
   float nt, nw;
   float2 pb[kLargePT / 2], pw[kLargePT / 2];  // B and w of the tile's outputs
+  __device__ __forceinline__ void tile_end(int i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      nt += __shfl_xor_sync(0xffffffffu, nt, o);
+      nw += __shfl_xor_sync(0xffffffffu, nw, o);
+    }
+    if ((threadIdx.x & 31) == 0) red[i * (kLargeNT / 32) + (threadIdx.x >> 5)] = make_float2(nt, nw);
+    nt = nw = 0.f;
+  }
+  __device__ __forceinline__ void row_end(int i, int lane) {
+    if (lane < kLargeNT / 32) red[i * (kLargeNT / 32) + lane] = make_float2(nt, nw);
+    nt = nw = 0.f;
+  }
   __device__ __forceinline__ void prefetch(int q, int k) {
     pb[q] = __ldg(B + k);
     pw[q] = w[k];
@@ -455,22 +583,29 @@ struct SnkTL {  // TL row: -10 log10 |u_n|^2 + 10 log10 r, n = 1..N
   float lr;
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
+  __device__ __forceinline__ void tile_end(int) {}
+  __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) {
     if (k >= 1) row[k - 1] = fmaf(-10.f, log10f(cabs2(v)), lr);
   }
 };
 
-template <int LOG2L>
+// The march: cluster blockIdx.x / NC marches solve descs[that].  The workspace is global memory, the tiles
+// and element-wise loops are shared out over the cluster's CTAs.
+template <int LOG2L, int NC>
 __global__ void __launch_bounds__(kLargeNT, 1)
     sssp_march_large_kernel(const SolveDesc* __restrict__ descs, const LargeTabs tb) {
   using C = CfgL<LOG2L>;
   constexpr int L = C::L;
   extern __shared__ __align__(16) float2 tile_smem[];
   __shared__ SolveDesc d;
-  __shared__ float red[2 * C::NW];
-  const int t = threadIdx.x;
+  constexpr int TILES = BigCfg<LOG2L>::CTAS, T = TILES / NC;  // tiles of a pass, and of this CTA
+  __shared__ float2 red[(TILES + 1) * C::NW];                 // norm partials of the stop test: per tile and warp,
+  __shared__ float2 part[TILES + 1];                          // per tile and for the odd row (every CTA's)
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int t = threadIdx.x, rank = int(cl.block_rank());
   {
-    const int* src = reinterpret_cast<const int*>(descs + blockIdx.x);
+    const int* src = reinterpret_cast<const int*>(descs + blockIdx.x / NC);
     int* dst = reinterpret_cast<int*>(&d);
     for (int i = t; i < int(sizeof(SolveDesc) / sizeof(int)); i += kLargeNT) dst[i] = src[i];
   }
@@ -490,20 +625,18 @@ __global__ void __launch_bounds__(kLargeNT, 1)
   double next_r = (node + 1 < d.nodes) ? d.node_r[node + 1] : 1e300;
   const float* V = iso ? nullptr : d.V + (size_t)node * L;
   const float* Vi = (iso || d.Vi == nullptr) ? nullptr : d.Vi + (size_t)node * L;
-  if (t == 0) {  // the zero mode is never visited by the transform's source
+  if (t == 0 && rank == 0) {  // the zero mode is never visited by the transform's source
     wsum[0] = make_float2(0.f, 0.f);
     t0[0] = make_float2(0.f, 0.f);
   }
   load_large_twiddles<LOG2L>(tile_smem, tb);
-  __syncthreads();
+  solve_sync<NC>();
+  const int i0 = t + rank * kLargeNT;  // element-wise loops: i = i0, i0 + NC kLargeNT, ...
 
   for (int s = 0; s < d.steps && status == kStatusOk; ++s) {
     if (iso) {
-      for (int q = 0; q < C::PER; ++q) {
-        const int i = t + q * kLargeNT;
-        y[i] = ffmul(__ldg(d.G + i), y[i]);
-      }
-      __syncthreads();
+      for (int i = i0; i < L; i += NC * kLargeNT) y[i] = ffmul(__ldg(d.G + i), y[i]);
+      solve_sync<NC>();
     } else {
       const double rmid = d.r0 + (double(s) + 0.5) * d.dr;
       if (rmid >= next_r) {
@@ -516,17 +649,38 @@ __global__ void __launch_bounds__(kLargeNT, 1)
         // t_0 = L_j^{-1} y in depth space; the source also sets t0 and w = t0 (spectral)
         {
           SnkArr sk{X};
-          dst_global<LOG2L>(W, tb, tile_smem, SrcStage{d.A + (size_t)j * L, y, t0, wsum}, sk);
+          dst_cluster<LOG2L, NC>(W, tile_smem, SrcStage{d.A + (size_t)j * L, y, t0, wsum}, sk, rank);
+          solve_sync<NC>();
         }
         ++ndst;
         float first = 0.f;
         for (int m = 1; m < d.terms; ++m) {
-          SnkTerm sk{d.B + (size_t)j * L, wsum, X, 0.f, 0.f, {}, {}};
-          dst_global<LOG2L>(W, tb, tile_smem, SrcV{X, V, Vi}, sk);  // B DST(V t_{m-1}), w += t_m
+          SnkTerm sk{d.B + (size_t)j * L, wsum, X, red, 0.f, 0.f, {}, {}};
+          dst_cluster<LOG2L, NC>(W, tile_smem, SrcV{X, V, Vi}, sk, rank);  // B DST(V t_{m-1}), w += t_m
           ++ndst;
-          const float snt = block_sum<LOG2L>(sk.nt, red);
-          const float snw = block_sum<LOG2L>(sk.nw, red + C::NW);
+          // (pass B ends with a block barrier) the totals of this CTA's tiles, to every CTA: summed per tile
+          // and then in tile order, so that the decision does not depend on the tiles' split over CTAs
+          constexpr int MINE = NC == 1 ? TILES + 1 : T;  // one CTA: its last tile is the odd row
+          auto total = [&](int c) {
+            float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int w = 0; w < C::NW; ++w) v = make_float2(v.x + red[c * C::NW + w].x, v.y + red[c * C::NW + w].y);
+            return v;
+          };
+          if constexpr (NC == 1) {
+            if (t < MINE) part[t] = total(t);
+          } else {
+            if (t < MINE * NC) cl.map_shared_rank(part, t / MINE)[rank * MINE + t % MINE] = total(t % MINE);
+            if (rank == NC - 1 && t >= kLargeNT - NC) cl.map_shared_rank(part, kLargeNT - 1 - t)[TILES] = total(TILES);
+          }
+          solve_sync<NC>();  // the term's results and every CTA's partials
           if (m == d.terms - 1) break;
+          float snt = 0.f, snw = 0.f;
+#pragma unroll
+          for (int c = 0; c <= TILES; ++c) {  // the same order in every CTA: a uniform decision
+            snt += part[c].x;
+            snw += part[c].y;
+          }
           if (!isfinite(snt) || !isfinite(snw)) {
             status = kStatusNumeric;
             break;
@@ -538,19 +692,17 @@ __global__ void __launch_bounds__(kLargeNT, 1)
           }
           if (neumann_stop_fast(snt, snw, d.tol2, tol2f)) break;
           SnkArr sx{X};
-          dst_global<LOG2L>(W, tb, tile_smem, SrcArr{X}, sx);  // t_m in depth space
+          dst_cluster<LOG2L, NC>(W, tile_smem, SrcArr{X}, sx, rank);  // t_m in depth space
+          solve_sync<NC>();
           ++ndst;
         }
         {
           const float4* rp = d.R + (size_t)j * L;
           const float2 bj = d.beta[j];
 #pragma unroll 4
-          for (int q = 0; q < C::PER; ++q) {
-            const int i = t + q * kLargeNT;
-            y[i] = ffmul(__ldg(rp + i), y[i]) + cmul(bj, wsum[i] - t0[i]);
-          }
+          for (int i = i0; i < L; i += NC * kLargeNT) y[i] = ffmul(__ldg(rp + i), y[i]) + cmul(bj, wsum[i] - t0[i]);
         }
-        __syncthreads();
+        solve_sync<NC>();
       }
       if (status != kStatusOk) break;
     }
@@ -558,20 +710,22 @@ __global__ void __launch_bounds__(kLargeNT, 1)
     if (d.tl_every > 0 && gs % d.tl_every == 0) {
       const float lr = float(10.0 * log10(d.r0 + double(s + 1) * d.dr));
       SnkTL sk{d.tl + (size_t)(d.rec0 + nrec) * d.N, lr};
-      dst_global<LOG2L>(W, tb, tile_smem, SrcScaled{y, out_scale}, sk);
+      dst_cluster<LOG2L, NC>(W, tile_smem, SrcScaled{y, out_scale}, sk, rank);
+      solve_sync<NC>();  // W is read out before the next transform writes it
       ++ndst;
       ++nrec;
     }
   }
   {  // physical envelope for pe_read_field
     SnkArr sk{d.field};
-    dst_global<LOG2L>(W, tb, tile_smem, SrcScaled{y, out_scale}, sk);
+    dst_cluster<LOG2L, NC>(W, tile_smem, SrcScaled{y, out_scale}, sk, rank);
     ++ndst;
   }
-  if (t == 0) {
+  if (t == 0 && rank == 0) {
     if (status != kStatusOk) atomicMax(d.status, status);
     atomicAdd(d.ndst, (unsigned long long)ndst);
   }
+  solve_sync<NC>();  // no CTA leaves while another may still write its partials
 }
 
 // One DST-I of a large grid: out = scale * DST(in); in holds N values, out L values.
@@ -588,6 +742,8 @@ struct SnkScaled {
   int off;
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
+  __device__ __forceinline__ void tile_end(int) {}
+  __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) {
     if (k + off > 0) out[k - 1 + off] = s * v;
   }

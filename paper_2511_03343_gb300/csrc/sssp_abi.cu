@@ -172,6 +172,10 @@ cudaError_t launch_dst_t(const float2* in, float2* out, float scale, const Trans
   return cudaGetLastError();
 }
 
+// CTAs that share a solve of the large-grid march, at most (the tiles of a pass)
+template <int LOG2L, int NC>
+constexpr int kLargeCtas = std::min(NC, sssp::BigCfg<LOG2L>::CTAS);
+
 // tables of the two-pass large-grid transform on the current device (cached per size)
 template <int LOG2L>
 cudaError_t large_tabs(sssp::LargeTabs* out) {
@@ -217,10 +221,10 @@ cudaError_t large_tabs(sssp::LargeTabs* out) {
   sssp::LargeTabs t{d, d + B::P, d + B::P + B::Q};
   cache[dev] = t;
   *out = t;
-  if ((e = cudaFuncSetAttribute(sssp::sssp_march_large_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(B::SMEM))) != cudaSuccess)
-    return e;
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  for (auto k : {sssp::sssp_march_large_kernel<LOG2L, kLargeCtas<LOG2L, 1>>, sssp::sssp_march_large_kernel<LOG2L, kLargeCtas<LOG2L, 2>>,
+                 sssp::sssp_march_large_kernel<LOG2L, kLargeCtas<LOG2L, 4>>})
+    if ((e = cudaFuncSetAttribute(k, at, int(B::SMEM_MARCH))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(sssp::sssp_dst_large_tile_kernel<LOG2L, false>, at, int(B::SMEM))) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(sssp::sssp_dst_large_tile_kernel<LOG2L, true>, at, int(B::SMEM))) != cudaSuccess) return e;
   return cudaFuncSetAttribute(sssp::sssp_dst_large_kernel<LOG2L>, at, int(B::SMEM));
@@ -231,13 +235,35 @@ cudaError_t large_tabs(sssp::LargeTabs* out) {
 // 48 / 32); the tiles' time grows with the fields once they fill the SMs, the other hardly before 64.
 constexpr int kLargeTileFields = 32;
 
+template <int LOG2L, int CTAS>
+cudaError_t launch_march_large_n(const SolveDesc* dDescs, int count, const sssp::LargeTabs& tb, cudaStream_t st) {
+  constexpr int NC = kLargeCtas<LOG2L, CTAS>;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = NC;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(unsigned(NC) * unsigned(count));
+  cfg.blockDim = dim3(sssp::kLargeNT);
+  cfg.dynamicSmemBytes = sssp::BigCfg<LOG2L>::SMEM_MARCH;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, sssp::sssp_march_large_kernel<LOG2L, NC>, dDescs, tb);
+}
+
+// As many CTAs a solve as the 152 SMs hold at once, up to 4 (the results do not depend on it).  N = 65535,
+// 2 steps, against one CTA a solve: 1 solve 14.0 -> 4.7 ms, 38 solves 15.0 -> 10.3, 76 solves 15.3 -> 11.2 (two CTAs
+// each); with 152 solves one CTA each takes 17.8, two or four 28 (an SM does a tile as fast, the barriers
+// and the single tiles' unhidden loads come on top).  N = 32767 1 solve 7.0 -> 2.3, N = 16383 8.2 -> 4.5 ms.
 template <int LOG2L>
 cudaError_t launch_march_large_t(const SolveDesc* dDescs, int count, const TransformTables&, cudaStream_t st) {
   sssp::LargeTabs tb;
   cudaError_t e = large_tabs<LOG2L>(&tb);
   if (e != cudaSuccess) return e;
-  sssp::sssp_march_large_kernel<LOG2L><<<count, sssp::kLargeNT, sssp::BigCfg<LOG2L>::SMEM, st>>>(dDescs, tb);
-  return cudaGetLastError();
+  if (count <= 38) return launch_march_large_n<LOG2L, 4>(dDescs, count, tb, st);
+  if (count <= 76) return launch_march_large_n<LOG2L, 2>(dDescs, count, tb, st);
+  return launch_march_large_n<LOG2L, 1>(dDescs, count, tb, st);
 }
 
 template <int LOG2L>

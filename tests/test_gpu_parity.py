@@ -1532,3 +1532,37 @@ def test_isovelocity_rows_split_over_ctas(sssp, N, bc, shape, count, steps, tl_e
             assert a[k].transform_count() == 2 * steps // tl_every + 2
     for p in a + b:
         p.close()
+
+
+# ----------------------------------------------------------------------------- large grids over several CTAs
+@pytest.mark.parametrize("N,counts", [(16383, (1, 77)), (32767, (1, 39, 77)), (65535, (1, 39, 77))])
+def test_large_march_same_bits_on_any_number_of_ctas(sssp, N, counts):
+    """The large-grid march shares a solve's tiles between 4, 2 or 1 CTAs, by how many solves a launch
+    holds: the same bits (field and TL row), transform count and stop decisions, with a real profile that
+    changes on the way, a complex one, and no profile at all."""
+    ref = None
+    for count in counts:
+        out = []
+        plans = []
+        for i in range(count):
+            s = inputs.munk(N=N, freq=300.0, dr=25.0, steps=3, pade_order=3, neumann_terms=(8, 6, 1)[i % 3] if count > 1 else 8)
+            n2 = s.profiles[0][1]
+            s.profiles = [(0.0, n2), (30.0, 1.0 + 0.8 * (n2 - 1.0))]
+            s.u0 = s.u0 + 0.3 * np.sin(np.pi * 40 * s.z / s.H) + 0.2j * np.sin(np.pi * 333 * s.z / s.H)
+            if i % 3 == 1:
+                s.profiles = [(0.0, n2 + 0.001j * (s.z / s.H) ** 2)]
+            pl = sssp.plan_for(s, tl_every=2)
+            pl.set_kernel("cta")
+            plans.append(pl)
+        sssp.march_batch(plans, 3)
+        for k in ((0,) if count == 1 else (0, 1, 2)):
+            out.append((plans[k].read_field(), plans[k].read_tl()[0], plans[k].transform_count()))
+        for pl in plans:
+            pl.close()
+        if ref is None:
+            ref = out
+        else:
+            for k in range(min(len(ref), len(out))):
+                assert np.array_equal(ref[k][0], out[k][0]) and np.array_equal(ref[k][1], out[k][1]) and ref[k][2] == out[k][2]
+            if len(out) > len(ref):
+                ref = out
