@@ -28,6 +28,7 @@
 // 40 steps: 9.1 -> 5.8 ms).  Its FP32 error is smaller too (no sums over L/2 modes): 3.1e-6 -> 1.2e-6
 // against complex128 there.
 #pragma once
+#include "march_dft.cuh"  // ldv2, ldv4
 #include "march_kernel.cuh"
 
 namespace sssp {
@@ -332,19 +333,6 @@ __device__ __forceinline__ void eo_forward(const float2 (&p)[4], const float2 (&
 #pragma unroll
     for (int i = 0; i < 4; ++i) sp[4 + i] = sp[4 + i] - x1[th.slot(i) + 1];
   }
-}
-
-// A stage's tables are read once a stage, at its ends, from the L2: the loads are issued together
-// (in program order, which volatile keeps) so that their latency is paid once.
-__device__ __forceinline__ float4 ldv4(const float4* p) {
-  float4 v;
-  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ float2 ldv2(const float2* p) {
-  float2 v;
-  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -17,6 +17,7 @@
 
 #include "../../include/sssp.h"
 #include "cluster_launch.h"
+#include "dft_launch.h"
 #include "eo_launch.h"
 #include "march_kernel.cuh"
 #include "march_large.cuh"
@@ -123,15 +124,16 @@ cudaError_t set_smem_attr() {
   if (done_dev == dev) return cudaSuccess;
   const int sm = int(Cfg<LOG2L>::SMEM), smc = int(Cfg<LOG2L>::SMEM_CPLX);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic>, a, sm);
   if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
-    e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet>, a, smc);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet>, a, sm);
   }
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic>, a, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic>, a, smc);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic>, a, sm);
+  if constexpr (!sssp_dft::supported(LOG2L)) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic>, a, sm);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic>, a, smc);
+  }
   if (e == cudaSuccess) done_dev = dev;
   return e;
 }
@@ -144,7 +146,8 @@ cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTa
   const int nt = Cfg<LOG2L>::NT;
   const size_t sm = Cfg<LOG2L>::SMEM, smc = Cfg<LOG2L>::SMEM_CPLX;
   if (bc == sssp::kBcPeriodic) {
-    if (cplx)
+    if constexpr (sssp_dft::supported(LOG2L)) return cudaErrorInvalidValue;  // the caller's other branch
+    else if (cplx)
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<dim3(count, split), nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
       sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<dim3(count, split), nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
@@ -304,6 +307,10 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
   // moves the transmission loss by up to 0.2 dB at its deepest nulls.
   if (bc == sssp::kBcDirichlet && sssp_eo::march_supported(log2L))
     return sssp_eo::launch_march(log2L, d, count, st, cplx);
+  // periodic, 512 .. 2048 points: the passes of march_dft.cuh (one solve of 512 points 1080 -> 890 cycles a
+  // transform, of 1024 1700 -> 1300, of 2048 3040 -> 2040; 300 of 2048 5640 -> 4290); below, a group of its threads would hold less than a row, and 4096 points need a longer one than a warp holds
+  if (bc == sssp::kBcPeriodic && sssp_dft::supported(log2L))
+    return sssp_dft::launch_march(log2L, d, count, st, cplx, split);
   switch (log2L) {
     case 3: return launch_march_t<3>(d, count, tabs, st, cplx, bc, split);
     case 4: return launch_march_t<4>(d, count, tabs, st, cplx, bc, split);
@@ -681,8 +688,9 @@ pe_status pe_plan_create_bc(pe_plan** out, int N, double H, double k0, double dr
   if (e != cudaSuccess) return bail(e, "cudaGetDevice");
   e = get_tables(p->device, log2L, &p->tabs);
   if (e != cudaSuccess) return bail(e, "transform tables");
-  if (bc == PE_BC_DIRICHLET && sssp_eo::supported(log2L) && (e = sssp_eo::prepare(log2L)) != cudaSuccess)
-    return bail(e, "parity-split kernel tables");
+  if (bc == PE_BC_DIRICHLET && sssp_eo::supported(log2L)) e = sssp_eo::prepare(log2L);
+  if (bc == PE_BC_PERIODIC && sssp_dft::supported(log2L)) e = sssp_dft::prepare(log2L);
+  if (e != cudaSuccess) return bail(e, "register transform tables");
   // plan tables in FP64 (Section 3: 1/(1 + b_j lambda_m), lambda_m = -(pi m/(k0 H))^2)
   const int L = p->L, P = pade_order;
   std::vector<float4> R(size_t(P) * L), G(L);

@@ -1566,3 +1566,30 @@ def test_large_march_same_bits_on_any_number_of_ctas(sssp, N, counts):
                 assert np.array_equal(ref[k][0], out[k][0]) and np.array_equal(ref[k][1], out[k][1]) and ref[k][2] == out[k][2]
             if len(out) > len(ref):
                 ref = out
+
+
+# ----------------------------------------------------------------------------- periodic grids of 512 .. 2048 points
+@pytest.mark.parametrize("N", [256, 512, 1024, 2048])
+@pytest.mark.parametrize("terms,absorb", [(1, False), (2, False), (12, False), (5, True)])
+def test_periodic_march_against_oracle(sssp, N, terms, absorb):
+    """The periodic march at every size of its register passes (one, two and four sub-rows a row) and the
+    size below, one, two, five and twelve terms, real and complex profiles with a node change, a TL row
+    every step, from a field with energy in every mode.  Bound as in test_parity_split_march_against_oracle."""
+    s = inputs.munk(N=N, freq=0.06 * N, dr=50.0 if N < 1000 else 25.0, steps=3, pade_order=4, neumann_terms=terms, bc="periodic")
+    rng = np.random.default_rng(N + terms)
+    l = np.minimum(np.arange(N), N - np.arange(N))
+    a = (rng.standard_normal(N) + 1j * rng.standard_normal(N)) / (1.0 + 16.0 * l / N) ** 2
+    s.u0 = np.fft.ifft(a) * N ** 0.5
+    n2 = s.profiles[0][1]
+    other = 1.0 + 0.9 * (n2 - 1.0) + 0.002 * np.sin(6.0 * np.pi * s.z / s.H)
+    if absorb:
+        other = other + 0.001j * (s.z / s.H) ** 2
+    s.profiles = [(0.0, n2.astype(other.dtype)), (1.5 * s.dr, other)]
+    u, tl, _, _ = _gpu(sssp, s)
+    if terms == 1:
+        s.profiles = [(0.0, np.ones(N))]
+    ref = _oracle(s)
+    assert np.linalg.norm(u - ref.u) / np.linalg.norm(ref.u) <= 12e-6 * math.log2(N) / 8
+    for k in range(s.steps):
+        got, want = 10.0 ** (-tl[k].astype(np.float64) / 20.0), 10.0 ** (-ref.tl[k] / 20.0)
+        assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 12e-6 * math.log2(N) / 8
