@@ -111,9 +111,14 @@ struct Cfg {
   static constexpr int MIN_BLOCKS = MB0 >= 16 ? 16 : (MB0 < 1 ? 1 : MB0);
   // dynamic shared memory: 2 padded buffers, twiddles, t_0 and B_j areas, sin weights, V row,
   // scan + reduce
-  static constexpr size_t SMEM = sizeof(float2) * (2 * PADL + 3 * L) + sizeof(float) * (2 * L) +
-                                 sizeof(float2) * NW + sizeof(float) * 2 * NW;
-  static constexpr size_t SMEM_CPLX = SMEM + sizeof(float) * L;  // + imaginary V row
+  static constexpr size_t SMEM0 = sizeof(float2) * (2 * PADL + 3 * L) + sizeof(float) * (2 * L) +
+                                  sizeof(float2) * NW + sizeof(float) * 2 * NW;
+  // Up to L = 512 a stage's tables are staged in shared memory ahead of their use (R where t_0 and B_j are
+  // otherwise, A and B in an area of their own) and the stop test rides on the next transform (StopHook):
+  // N = 255 1400 -> 1300 cycles a transform.  At L = 1024 one solve gained 1 %, 256 solves lost 1 %.
+  static constexpr bool AHEAD = OPREG && L <= 512;
+  static constexpr size_t SMEM = SMEM0 + (AHEAD ? sizeof(float4) * L : 0);
+  static constexpr size_t SMEM_CPLX = AHEAD ? SMEM : SMEM0 + sizeof(float) * L;  // + imaginary V row
 };
 
 // padded shared-memory index: one pad element per 16 (128 B), so contiguous half-warp
@@ -454,13 +459,20 @@ __device__ __forceinline__ float2* fft_rest(float2* src, float2* dst, const floa
   }
 }
 
+// Work a transform takes along on its first barrier: publish() before it, and stop() after it, which may
+// end the transform there (every thread the same way).
+struct NoHook {
+  __device__ __forceinline__ void publish() {}
+  __device__ __forceinline__ bool stop() { return false; }
+};
+
 // Unnormalised DST-I of the L values in `a` (natural order, padded; a[0] is ignored) into
 // out[0..P) = S_{P t..P t+P) of thread t (S_0 = 0).  Uses `b` as the ping-pong buffer.
-// On return every thread has finished reading both buffers.
-template <int LOG2L, int PPT = 8>
-__device__ __forceinline__ void dst_block(float2* a, float2* b, const float2* __restrict__ tw,
+// On return every thread has finished reading both buffers.  False: the hook ended it.
+template <int LOG2L, int PPT = 8, class HOOK = NoHook>
+__device__ __forceinline__ bool dst_block(float2* a, float2* b, const float2* __restrict__ tw,
                                           const float* __restrict__ sinw, float2* scan_s, float2 (&out)[PPT],
-                                          const TwRegs<LOG2L, PPT>* twr = nullptr) {
+                                          const TwRegs<LOG2L, PPT>* twr = nullptr, HOOK hook = {}) {
   using C = Cfg<LOG2L, PPT>;
   constexpr int L = C::L, H = C::HALF;
   const int t = threadIdx.x;
@@ -478,7 +490,9 @@ __device__ __forceinline__ void dst_block(float2* a, float2* b, const float2* __
 #pragma unroll
     for (int r = 0; r < PPT; ++r) b[pidx(PPT * t + r)] = v[r];
   }
+  hook.publish();
   __syncthreads();
+  if (hook.stop()) return false;
   // When the passes end with radix 2 (span L/2), that pass is fused into the post-processing:
   // with the earlier passes' result F and w = e^{-2 pi i/L}, Y_k = F_k + w^k F_{k+L/2} and
   // Y_{L-k} = F_{L/2-k} + conj(w^k) F_{L-k} (the butterfly of L/2 - k, whose twiddle is
@@ -531,6 +545,7 @@ __device__ __forceinline__ void dst_block(float2* a, float2* b, const float2* __
     out[2 * s] = se[s];
     out[2 * s + 1] = dd[s] + excl;
   }
+  return true;
 }
 
 // Boundary conditions of Section 3.1: homogeneous Dirichlet (DST-I, the workloads) and
@@ -541,8 +556,9 @@ constexpr int kBcPeriodic = 1;
 // Unnormalised DFT of the L values in `a` (natural order, padded) into out[0..P) = X_{Pt..Pt+P)
 // of thread t; INV uses e^{+2 pi i n m/L} (by conjugating input and output).  On return every
 // thread has finished reading both buffers.
-template <int LOG2L, bool INV, int PPT = 8>
-__device__ __forceinline__ void dft_block(float2* a, float2* b, const float2* __restrict__ tw, float2 (&out)[PPT]) {
+template <int LOG2L, bool INV, int PPT = 8, class HOOK = NoHook>
+__device__ __forceinline__ bool dft_block(float2* a, float2* b, const float2* __restrict__ tw, float2 (&out)[PPT],
+                                          HOOK hook = {}) {
   constexpr int L = 1 << LOG2L;
   const int t = threadIdx.x;
   {
@@ -556,7 +572,9 @@ __device__ __forceinline__ void dft_block(float2* a, float2* b, const float2* __
 #pragma unroll
     for (int r = 0; r < PPT; ++r) b[pidx(PPT * t + r)] = v[r];
   }
+  hook.publish();
   __syncthreads();
+  if (hook.stop()) return false;
   const float2* F = fft_rest<LOG2L, PPT, PPT>(b, a, tw);
 #pragma unroll
   for (int i = 0; i < PPT; ++i) {
@@ -564,20 +582,79 @@ __device__ __forceinline__ void dft_block(float2* a, float2* b, const float2* __
     out[i] = INV ? conjf2(x) : x;
   }
   __syncthreads();
+  return true;
 }
 
 // The transform of the boundary condition: TO_DEPTH maps spectral coefficients to depth values
 // (the inverse transform up to the scale folded into the tables), otherwise depth -> spectral.
-template <int LOG2L, int BC, bool TO_DEPTH, int PPT = 8>
-__device__ __forceinline__ void xform(float2* a, float2* b, const float2* __restrict__ tw,
+template <int LOG2L, int BC, bool TO_DEPTH, int PPT = 8, class HOOK = NoHook>
+__device__ __forceinline__ bool xform(float2* a, float2* b, const float2* __restrict__ tw,
                                       const float* __restrict__ sinw, float2* scan_s, float2 (&out)[PPT],
-                                      const TwRegs<LOG2L, PPT>* twr = nullptr) {
+                                      const TwRegs<LOG2L, PPT>* twr = nullptr, HOOK hook = {}) {
   if constexpr (BC == kBcPeriodic) {
-    dft_block<LOG2L, TO_DEPTH, PPT>(a, b, tw, out);
+    return dft_block<LOG2L, TO_DEPTH, PPT>(a, b, tw, out, hook);
   } else {
-    dst_block<LOG2L, PPT>(a, b, tw, sinw, scan_s, out, twr);  // DST-I is its own inverse
+    return dst_block<LOG2L, PPT>(a, b, tw, sinw, scan_s, out, twr, hook);  // DST-I is its own inverse
   }
 }
+
+// The stop test of the Neumann series.  As a hook it rides on the next (inverse) transform's first barrier:
+// the warps reduce their norm partials while the transform's first pass runs, and the decision is taken one
+// pass into it -- a pass wasted once a stage, against the reduction's chain of shuffles every term.
+template <int WS, int NW, unsigned MASK>
+struct StopHook {
+  float nt, nw;  // this thread's partials
+  float* red;
+  int m;         // the term tested
+  float* first;
+  int* status;
+  double tol2;
+  float tol2f;
+  __device__ __forceinline__ void publish() {
+#pragma unroll
+    for (int o = WS / 2; o > 0; o >>= 1) {
+      nt += __shfl_xor_sync(MASK, nt, o, WS);
+      nw += __shfl_xor_sync(MASK, nw, o, WS);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      red[2 * (threadIdx.x >> 5)] = nt;
+      red[2 * (threadIdx.x >> 5) + 1] = nw;
+    }
+  }
+  __device__ __forceinline__ bool stop() {
+    // block totals: every thread adds the warps' partials in the same order (broadcast
+    // reads, no dependent shuffles), so EVERY thread holds the same total — the stop
+    // decision below must be uniform across the block (it guards __syncthreads).
+    float snt = 0.f, snw = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      const float2 pr = reinterpret_cast<const float2*>(red)[w];
+      snt += pr.x;
+      snw += pr.y;
+    }
+    if (!isfinite(snt) || !isfinite(snw)) {
+      *status = kStatusNumeric;
+      return true;
+    }
+    // blow-up: a term 1e4 times the first correction term.  (Growth over a few terms
+    // alone is no evidence: the operator b_j L_j^{-1} V is not normal, so convergent
+    // series can grow transiently.)
+    if (m == 1) *first = snt;
+    else if (*first > 0.f && snt > 1e8f * *first) {
+      *status = kStatusDiverged;
+      return true;
+    }
+    return neumann_stop_fast(snt, snw, tol2, tol2f);
+  }
+};
+
+// 16 bytes global -> shared, asynchronously; the thread's own copies only, waited for by group
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(unsigned(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 template <int LOG2L, int PPT = 8>
 __device__ __forceinline__ void load_tables(float2* tw, float* sinw, const float2* __restrict__ tw_g,
@@ -614,6 +691,9 @@ struct Smem {
     red = reinterpret_cast<float*>(scan_s + C::NW);
     Vis = red + 2 * C::NW;  // only present in the complex-profile kernel (SMEM_CPLX)
   }
+  // the tables staged ahead (Cfg::AHEAD)
+  __device__ __forceinline__ float4* stage_r() const { return reinterpret_cast<float4*>(t0s); }
+  __device__ __forceinline__ float4* stage_ab() const { return reinterpret_cast<float4*>(Vis); }
 };
 
 // P consecutive complex values of one thread, 16-byte vector accesses (P even, p 16-byte aligned)
@@ -671,7 +751,6 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
   Smem<LOG2L, PPT> sm(smem_raw);
   __shared__ SolveDesc d;
   const int t = threadIdx.x;
-  const int lane = t & 31, warp = t >> 5;
   {  // the descriptor lives in shared memory so its fields need no registers
     const int* src = reinterpret_cast<const int*>(descs + blockIdx.x);
     int* dst = reinterpret_cast<int*>(&d);
@@ -721,6 +800,21 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
     }
   };
   if (!iso) load_v(node);
+  // Tables staged a stage ahead (A and B) or over the stage (R): each thread copies the entries of its own
+  // modes, so no barrier is involved.
+  auto stage_ab = [&](int j) {
+    const float4* A = reinterpret_cast<const float4*>(d.A + (size_t)j * L + P * t);
+    const float4* B = reinterpret_cast<const float4*>(d.B + (size_t)j * L + P * t);
+#pragma unroll
+    for (int i = 0; i < P / 2; ++i) {
+      cp_async16(sm.stage_ab() + i * C::NT + t, A + i);
+      cp_async16(sm.stage_ab() + (P / 2 + i) * C::NT + t, B + i);
+    }
+    cp_async_commit();
+  };
+  if constexpr (C::AHEAD) {
+    if (!iso) stage_ab(0);
+  }
   __syncthreads();
 
   if (iso) {
@@ -766,14 +860,24 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
       for (int j = 0; j < d.p && status == kStatusOk; ++j) {
         float2 acc[P], tp[P];
         float2 Bj[P], t0r[P];  // register copies of B_j and t_0 (OPREG), else in sm.Bs / sm.t0s
-        load8<LOG2L, P>(d.B + (size_t)j * L + P * t, Bj);
-        if constexpr (!C::OPREG) {
-#pragma unroll
-          for (int i = 0; i < P; ++i) sm.Bs[i * C::NT + t] = Bj[i];
-        }
         {
           float2 Aj[P];
-          load8<LOG2L, P>(d.A + (size_t)j * L + P * t, Aj);
+          if constexpr (C::AHEAD) {
+            cp_async_wait<0>();
+#pragma unroll
+            for (int i = 0; i < P / 2; ++i) {
+              const float4 a = sm.stage_ab()[i * C::NT + t], b = sm.stage_ab()[(P / 2 + i) * C::NT + t];
+              Aj[2 * i] = make_float2(a.x, a.y), Aj[2 * i + 1] = make_float2(a.z, a.w);
+              Bj[2 * i] = make_float2(b.x, b.y), Bj[2 * i + 1] = make_float2(b.z, b.w);
+            }
+          } else {
+            load8<LOG2L, P>(d.B + (size_t)j * L + P * t, Bj);
+            if constexpr (!C::OPREG) {
+#pragma unroll
+              for (int i = 0; i < P; ++i) sm.Bs[i * C::NT + t] = Bj[i];
+            }
+            load8<LOG2L, P>(d.A + (size_t)j * L + P * t, Aj);
+          }
 #pragma unroll
           for (int i = 0; i < P; ++i) {
             const float2 t0 = cmul(Aj[i], y[i]);
@@ -784,6 +888,12 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
           }
         }
         __syncthreads();
+        if constexpr (C::AHEAD) {  // R_j for this stage's end, then A and B of the next stage
+#pragma unroll
+          for (int i = 0; i < P; ++i) cp_async16(sm.stage_r() + i * C::NT + t, d.R + (size_t)j * L + P * t + i);
+          cp_async_commit();
+          stage_ab(j + 1 < d.p ? j + 1 : 0);
+        }
         xform<LOG2L, BC, true, P>(sm.bufA, sm.bufB, sm.tw, sm.sinw, sm.scan_s, tp, twr);  // t_0 in depth space
         ++ndst;
         float first = 0.f;
@@ -810,53 +920,29 @@ __global__ void __launch_bounds__(Cfg<LOG2L, PPT>::NT, Cfg<LOG2L, PPT>::MIN_BLOC
             nt += cabs2(tp[i]);
             nw += cabs2((C::OPREG ? t0r[i] : sm.t0s[i * C::NT + t]) + acc[i]);
           }
+          if (m == d.terms - 1) break;
 #pragma unroll
-          for (int o = C::WS / 2; o > 0; o >>= 1) {
-            nt += __shfl_xor_sync(C::MASK, nt, o, C::WS);
-            nw += __shfl_xor_sync(C::MASK, nw, o, C::WS);
+          for (int i = 0; i < P; ++i) sm.bufA[pidx(P * t + i)] = tp[i];
+          // t_m in depth space, unless its stop test ends the series
+          StopHook<C::WS, C::NW, C::MASK> hook{nt, nw, sm.red, m, &first, &status, d.tol2, tol2f};
+          if constexpr (C::AHEAD) {
+            __syncthreads();
+            if (!xform<LOG2L, BC, true, P>(sm.bufA, sm.bufB, sm.tw, sm.sinw, sm.scan_s, tp, twr, hook)) break;
+          } else {
+            hook.publish();
+            __syncthreads();
+            if (hook.stop()) break;
+            xform<LOG2L, BC, true, P>(sm.bufA, sm.bufB, sm.tw, sm.sinw, sm.scan_s, tp, twr);
           }
-          if (lane == 0) {
-            sm.red[2 * warp] = nt;
-            sm.red[2 * warp + 1] = nw;
-          }
-          const bool last = (m == d.terms - 1);
-          if (!last) {
-#pragma unroll
-            for (int i = 0; i < P; ++i) sm.bufA[pidx(P * t + i)] = tp[i];
-          }
-          __syncthreads();
-          if (last) break;
-          // block totals: every thread adds the warps' partials in the same order (broadcast
-          // reads, no dependent shuffles), so EVERY thread holds the same total — the stop
-          // decision below must be uniform across the block (it guards __syncthreads).
-          float snt = 0.f, snw = 0.f;
-#pragma unroll
-          for (int w = 0; w < C::NW; ++w) {
-            const float2 pr = reinterpret_cast<const float2*>(sm.red)[w];
-            snt += pr.x;
-            snw += pr.y;
-          }
-          if (!isfinite(snt) || !isfinite(snw)) {
-            status = kStatusNumeric;
-            break;
-          }
-          // blow-up: a term 1e4 times the first correction term.  (Growth over a few terms
-          // alone is no evidence: the operator b_j L_j^{-1} V is not normal, so convergent
-          // series can grow transiently.)
-          if (m == 1) first = snt;
-          else if (first > 0.f && snt > 1e8f * first) {
-            status = kStatusDiverged;
-            break;
-          }
-          if (neumann_stop_fast(snt, snw, d.tol2, tol2f)) break;
-          xform<LOG2L, BC, true, P>(sm.bufA, sm.bufB, sm.tw, sm.sinw, sm.scan_s, tp, twr);  // t_m in depth space
           ++ndst;
         }
         {
           const float4* rp = d.R + (size_t)j * L + P * t;
           const float2 bj = d.beta[j];
+          if constexpr (C::AHEAD) cp_async_wait<1>();
 #pragma unroll
-          for (int i = 0; i < P; ++i) y[i] = ffmul(__ldg(rp + i), y[i]) + cmul(bj, acc[i]);
+          for (int i = 0; i < P; ++i)
+            y[i] = ffmul(C::AHEAD ? sm.stage_r()[i * C::NT + t] : __ldg(rp + i), y[i]) + cmul(bj, acc[i]);
         }
       }
       if (status != kStatusOk) break;

@@ -167,10 +167,10 @@ cudaError_t launch_dst_t(const float2* in, float2* out, float scale, const Trans
   cudaError_t e = set_smem_attr<LOG2L>();
   if (e != cudaSuccess) return e;
   if (bc == sssp::kBcPeriodic)
-    sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
+    sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM0, st>>>(
         in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
   else if constexpr (LOG2L < sssp_eo::kMinMarchLog2)
-    sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM, st>>>(
+    sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM0, st>>>(
         in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
   return cudaGetLastError();
 }

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(sssp::Cfg<LOG2L>::NT)
 template <int LOG2L>
 cudaError_t noalloc_attr() {
   return cudaFuncSetAttribute(sssp_noalloc_dst_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(sssp::Cfg<LOG2L>::SMEM));
+                              int(sssp::Cfg<LOG2L>::SMEM0));
 }
 
 template <int LOG2L>
@@ -97,7 +97,7 @@ cudaError_t noalloc_launch(const NoAllocDevice& d, cudaStream_t st) {
   constexpr int L = 1 << LOG2L;
   const float2* tw = d.tw + (L - 8);
   const float* sw = d.sinw + (L - 8);
-  sssp_noalloc_dst_kernel<LOG2L><<<1, sssp::Cfg<LOG2L>::NT, sssp::Cfg<LOG2L>::SMEM, st>>>(
+  sssp_noalloc_dst_kernel<LOG2L><<<1, sssp::Cfg<LOG2L>::NT, sssp::Cfg<LOG2L>::SMEM0, st>>>(
       d.scratch, d.scratch + kNoAllocMaxL, tw, sw);
   return cudaGetLastError();
 }
