@@ -51,6 +51,7 @@ struct pe_plan {
   int nodes = 0, node_cap = 0;
   std::vector<double> node_r;
   int* dStatus = nullptr;
+  int* hStatus = nullptr;    // its landing place in pinned host memory (null: none was free)
   unsigned long long* dNdst = nullptr;
   float* dTL = nullptr;
   long long tl_cap_rows = 0, tl_rows = 0;

@@ -82,6 +82,43 @@ cudaError_t get_tables(int device, int log2L, TransformTables* out, int ppt = 8)
   return cudaSuccess;
 }
 
+// Pinned host words the plans' status words are copied to: a copy to pageable memory is staged and waited
+// for by the runtime, one to pinned memory is one more item of the stream (or a kernel's store), and the
+// call's own synchronisation covers it.  One page for all plans of the process, taken with the first plan
+// and given back with the last; a plan that finds none free copies to pageable memory.
+struct StatusSlots {
+  static constexpr int kSlots = 1024;
+  std::mutex mu;
+  int* base = nullptr;
+  std::vector<int*> free;
+  int* take() {
+    std::lock_guard<std::mutex> lk(mu);
+    if (!base) {
+      if (cudaHostAlloc(reinterpret_cast<void**>(&base), kSlots * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) !=
+          cudaSuccess) {
+        cudaGetLastError();
+        base = nullptr;
+        return nullptr;
+      }
+      for (int i = kSlots; i-- > 0;) free.push_back(base + i);
+    }
+    if (free.empty()) return nullptr;
+    int* s = free.back();
+    free.pop_back();
+    return s;
+  }
+  void give(int* s) {
+    if (!s) return;
+    std::lock_guard<std::mutex> lk(mu);
+    free.push_back(s);
+    if (int(free.size()) < kSlots) return;
+    cudaFreeHost(base);
+    base = nullptr;
+    free.clear();
+  }
+};
+StatusSlots g_status_slots;
+
 int ilog2_exact(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
@@ -364,8 +401,9 @@ __global__ void even_extend_kernel(float2* buf, int K) {
 }
 
 __global__ void carrier_kernel(const float2* __restrict__ field, float2* __restrict__ out, float c, float s, int N,
-                               int off) {
+                               int off, const int* status, int* host_status) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n == 0 && host_status) *host_status = *status;
   if (n < N) {
     const float2 v = field[n + off];
     out[n] = make_float2(c * v.x - s * v.y, c * v.y + s * v.x);
@@ -543,10 +581,14 @@ int group_iso_rows(const std::vector<SolveDesc>& g) {
   return rows;
 }
 
-pe_status check_status(pe_plan* p) {
+// Wait for the plan's stream and report the device's status word; `copied`: a kernel of the stream has
+// already stored it to the plan's pinned word
+pe_status check_status(pe_plan* p, bool copied = false) {
   int s = 0;
-  PE_CUDA(p, cudaMemcpyAsync(&s, p->dStatus, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+  int* to = p->hStatus ? p->hStatus : &s;
+  if (!copied || !p->hStatus) PE_CUDA(p, cudaMemcpyAsync(to, p->dStatus, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
   PE_CUDA(p, cudaStreamSynchronize(p->stream));
+  s = *const_cast<volatile int*>(to);
   if (s == sssp::kStatusDiverged)
     return fail(p, PE_ERR_NEUMANN_DIVERGED, "Neumann series diverged (a term grew to 1e4 times the first correction)");
   if (s == sssp::kStatusNumeric) return fail(p, PE_ERR_NUMERIC, "non-finite value in the march");
@@ -600,6 +642,7 @@ void pe_plan_destroy(pe_plan* p) {
   cudaFree(p->dVi);
   cudaFree(p->dNodeR);
   cudaFree(p->dStatus);
+  g_status_slots.give(p->hStatus);
   cudaFree(p->dNdst);
   cudaFree(p->dTL);
   cudaFree(p->dDesc);
@@ -740,6 +783,7 @@ pe_status pe_plan_create_bc(pe_plan** out, int N, double H, double k0, double dr
   if ((e = cudaMalloc(&p->dField, sizeof(float2) * L)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = cudaMalloc(&p->dStage, sizeof(float2) * L)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = cudaMalloc(&p->dStatus, sizeof(int))) != cudaSuccess) return bail(e, "cudaMalloc");
+  p->hStatus = g_status_slots.take();
   if (log2L > kMaxSmemLog2 &&
       (e = cudaMalloc(&p->dWork, sizeof(float2) * sssp::large_work_elems(L))) != cudaSuccess)
     return bail(e, "cudaMalloc(workspace)");
@@ -1118,12 +1162,12 @@ pe_status pe_read_field(pe_plan* p, float* out, int to_device) {
   const float c = float(std::cos(phase)), s = float(std::sin(phase));
   const bool direct = to_device && p->N_user == p->N;
   float2* dst = direct ? reinterpret_cast<float2*>(out) : p->dStage;
-  carrier_kernel<<<(p->N + 255) / 256, 256, 0, p->stream>>>(p->dField, dst, c, s, p->N, p->off);
+  carrier_kernel<<<(p->N + 255) / 256, 256, 0, p->stream>>>(p->dField, dst, c, s, p->N, p->off, p->dStatus, p->hStatus);
   PE_CUDA(p, cudaGetLastError());
   if (!direct)
     PE_CUDA(p, cudaMemcpyAsync(out, p->dStage, sizeof(float2) * p->N_user,
                                to_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, p->stream));
-  return check_status(p);
+  return check_status(p, true);
 }
 
 pe_status pe_read_TL(pe_plan* p, float* out, size_t cap, double* ranges, size_t* n_rows) {
@@ -1133,7 +1177,9 @@ pe_status pe_read_TL(pe_plan* p, float* out, size_t cap, double* ranges, size_t*
   if (n_rows) *n_rows = size_t(p->tl_rows);
   if (!out) return PE_OK;  // size query
   if (cap < need) return fail(p, PE_ERR_ARG, "TL buffer too small");
-  if (need > 0)  // rows hold N values on the device; the caller gets the first N_user of each
+  if (need > 0 && p->N_user == p->N)  // the rows as they lie
+    PE_CUDA(p, cudaMemcpyAsync(out, p->dTL, sizeof(float) * need, cudaMemcpyDeviceToHost, p->stream));
+  else if (need > 0)  // rows hold N values on the device; the caller gets the first N_user of each
     PE_CUDA(p, cudaMemcpy2DAsync(out, sizeof(float) * p->N_user, p->dTL, sizeof(float) * p->N,
                                  sizeof(float) * p->N_user, size_t(p->tl_rows), cudaMemcpyDeviceToHost, p->stream));
   if (ranges)
