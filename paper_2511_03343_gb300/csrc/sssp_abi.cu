@@ -1098,11 +1098,7 @@ pe_status pe_march_batch_steps(pe_plan** plans, const int* steps, int count) {
   PE_CUDA(p0, lanes_for(p0->device, int(groups.size()), &bl));
   PE_CUDA(p0, cudaEventRecord(bl->fork, p0->stream));
   int g = 0;
-  // Largest grids first: a cluster needs its SMs free at once, which the CTAs of small grids scattered over
-  // the device do not leave, while those fit beside it.  45 solves of N = 255 .. 8191, 9 of each:
-  // 15.2 -> 11.1 ms, the time of the N = 8191 solves alone.
-  for (auto it = groups.rbegin(); it != groups.rend(); ++it) {
-    auto& kv = *it;
+  for (auto& kv : groups) {
     cudaStream_t st = bl->streams[g];
     const size_t bytes = sizeof(SolveDesc) * kv.second.size();
     PE_CUDA(p0, cudaStreamWaitEvent(st, bl->fork, 0));
