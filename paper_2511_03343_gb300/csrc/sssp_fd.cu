@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 
 #include <complex>
+#include <mutex>
+#include <set>
 #include <vector>
 
 #include "fd_launch.h"
@@ -14,7 +16,21 @@ namespace {
 
 template <int LOG2L>
 cudaError_t launch_t(const sssp::SolveDesc* d, int count, cudaStream_t st) {
-  sssp::sssp_fd_march_kernel<LOG2L><<<count, sssp::FdCfg<LOG2L>::NT, 0, st>>>(d);
+  using C = sssp::FdCfg<LOG2L>;
+  static std::mutex mu;
+  static std::set<int> done;  // devices whose shared-memory attribute is set
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (!done.count(dev)) {
+      e = cudaFuncSetAttribute(sssp::sssp_fd_march_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+      if (e != cudaSuccess) return e;
+      done.insert(dev);
+    }
+  }
+  sssp::sssp_fd_march_kernel<LOG2L><<<count, C::NT, C::SMEM, st>>>(d);
   return cudaGetLastError();
 }
 

@@ -1593,3 +1593,21 @@ def test_periodic_march_against_oracle(sssp, N, terms, absorb):
     for k in range(s.steps):
         got, want = 10.0 ** (-tl[k].astype(np.float64) / 20.0), 10.0 ** (-ref.tl[k] / 20.0)
         assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 12e-6 * math.log2(N) / 8
+
+
+@pytest.mark.parametrize("N,p", [(7, 1), (63, 3), (1023, 8), (2047, 2)])
+def test_fdssp_staged_tables_against_oracle(sssp, N, p):
+    """The FD-SSP march's tables staged ahead: one thread, a partial warp, the largest staged grid, one
+    stage and eight, with a profile node per step (the next step's table is fetched during the last stage)."""
+    s = inputs.munk(N=N, freq=0.02 * (N + 1) + 2.0, dr=50.0, steps=7, pade_order=p)
+    n = np.arange(1, N + 1)
+    s.u0 = sum(np.sin(np.pi * n * m / (N + 1)) * (1.0 + 0.5j * m) / m for m in range(1, min(N, 9) + 1))
+    n2 = s.profiles[0][1]
+    s.profiles = [(k * s.dr, 1.0 + (1.0 + 0.02 * k) * (n2 - 1.0)) for k in range(s.steps)]
+    pl = sssp.plan_for(s, tl_every=3, op="fd3")
+    pl.march(3)
+    pl.march(s.steps - 3)
+    u = pl.read_field()
+    tl, _ = pl.read_tl()
+    pl.close()
+    _compare(u, tl, _fd_oracle(s, 3))
