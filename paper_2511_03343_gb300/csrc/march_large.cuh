@@ -1,6 +1,5 @@
 // SSSP range march for grids larger than one CTA's shared memory (L = N + 1 = 8192 .. 65536).
 //
-// A solve is marched by a cluster of 1, 2 or 4 CTAs that share its tiles.
 // Same method as march_kernel.cuh (product-form Pade stages with hi/lo multipliers, Neumann
 // series, spectral-resident field), but every length-L array lives in a per-solve workspace
 // in global memory (L2-resident for a few solves, HBM for large batches).  CTAs of 512 threads, one per
