@@ -924,7 +924,7 @@ def bench_munk(args):
                 "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                              "frac": achieved / peak, "traffic": None,
                              "kernel": ("sssp_march_cluster_kernel<12, 8> (one solve over an 8-CTA cluster, 8 SMs)"
-                                        if pl.kernel == "cluster" else "sssp_march_kernel<12> (one CTA, one SM)"),
+                                        if pl.kernel == "cluster" else "sssp_march_eo_kernel<12> (one CTA, one SM)"),
                              "flops_per_launch": flops, "dst_per_launch": dst_per_launch,
                              "kernel_ms": kern_avg,
                              "peak_note": f"FP32 FMA peak of all {sms} SMs at the sampled max SM clock (derived, not measured)"},

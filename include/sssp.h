@@ -203,7 +203,7 @@ pe_status pe_get_transform_count(pe_plan* plan, unsigned long long* count);
 pe_status pe_dst1(pe_plan* plan, const float* in, float* out, int on_device);
 
 /*
- * `count` DST-I of length N at once (one CTA per field), in and out device memory holding
+ * `count` DST-I of length N at once, in and out device memory holding
  * count x N interleaved complex64 values (row b = field b).  Asynchronous on the plan's
  * stream.  Section 3.1's transform, batched.
  */
@@ -284,7 +284,8 @@ pe_status pe_plan_set_operator(pe_plan* plan, int op);
 /*
  * Shape of the one-CTA shared-memory kernel (no counterpart in the paper): points per thread
  * P = 4, 8 (default; 0 means 8) or 16, i.e. L/P threads per solve, each transform a Stockham FFT
- * of radix-P passes.  4 and 16 take Dirichlet grids with N + 1 in [256, 4096]; PE_ERR_ARG
+ * of radix-P passes (at 8 points, N + 1 = 2048 and 4096 run the kernel that splits the modes by
+ * parity).  4 and 16 take Dirichlet grids with N + 1 in [256, 4096]; PE_ERR_ARG
  * otherwise.  All shapes compute the same step (results agree to FP32 rounding).
  * pe_plan_get_shape reports the P a march of the plan runs (0 when it runs the cluster or the
  * large-grid kernel).
