@@ -446,7 +446,7 @@ __device__ __forceinline__ void dst_last_row(const float2* W, float2* sm, SNK& s
       snk.put(0, k, make_float2(-0.5f * zk.y, 0.5f * zk.x));
     }
   }
-  snk.row_end(C::CTAS, lane);
+  snk.template row_end<G>(C::CTAS, lane);
   __syncwarp();
 }
 
@@ -522,13 +522,14 @@ struct SrcScaled {  // x_m = s y_m
 };
 // A sink takes put(q, k, S_k) for its q-th output of a tile; prefetch(q, k) is called for the
 // same (q, k) before the tile's FFT, so a sink can load its own operands early; tile_end(i) after the
-// thread's last output of the i-th tile of its CTA, row_end(CTAS, lane) after the odd row of a cluster's march.
+// thread's last output of the i-th tile of its CTA, row_end<G>(CTAS, lane) after the odd row of a cluster's march.
 struct SnkArr {
   static constexpr bool kL2 = false;  // write-only: no operands to fetch
   float2* a;
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
   __device__ __forceinline__ void tile_end(int) {}
+  template <int>
   __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) { a[k] = v; }
 };
@@ -555,8 +556,17 @@ struct SnkTerm {  // t_m = B_k S_k: w += t_m, X = t_m, and the norm partials of 
     if ((threadIdx.x & 31) == 0) red[i * (kLargeNT / 32) + (threadIdx.x >> 5)] = make_float2(nt, nw);
     nt = nw = 0.f;
   }
+  // The odd row's partials, lane i < G holding the outputs i + G q.  A tile of TR rows gives these to the
+  // threads i TR + TR - 1, G / 16 of them in a warp, whose sum is the warp's slot.
+  template <int G>
   __device__ __forceinline__ void row_end(int i, int lane) {
-    if (lane < kLargeNT / 32) red[i * (kLargeNT / 32) + lane] = make_float2(nt, nw);
+    static_assert(G <= kLargeNT / 32 || G == kLargeNT / 16, "at most two of a row's threads in a warp");
+    constexpr int PER = G == kLargeNT / 16 ? 2 : 1;
+    if constexpr (PER == 2) {
+      nt += __shfl_xor_sync(0xffffffffu, nt, 1);
+      nw += __shfl_xor_sync(0xffffffffu, nw, 1);
+    }
+    if (lane % PER == 0 && lane / PER < kLargeNT / 32) red[i * (kLargeNT / 32) + lane / PER] = make_float2(nt, nw);
     nt = nw = 0.f;
   }
   __device__ __forceinline__ void prefetch(int q, int k) {
@@ -583,6 +593,7 @@ struct SnkTL {  // TL row: -10 log10 |u_n|^2 + 10 log10 r, n = 1..N
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
   __device__ __forceinline__ void tile_end(int) {}
+  template <int>
   __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) {
     if (k >= 1) row[k - 1] = fmaf(-10.f, log10f(cabs2(v)), lr);
@@ -742,6 +753,7 @@ struct SnkScaled {
   __device__ __forceinline__ void l2(int) {}
   __device__ __forceinline__ void prefetch(int, int) {}
   __device__ __forceinline__ void tile_end(int) {}
+  template <int>
   __device__ __forceinline__ void row_end(int, int) {}
   __device__ __forceinline__ void put(int, int k, float2 v) {
     if (k + off > 0) out[k - 1 + off] = s * v;

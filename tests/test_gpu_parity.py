@@ -1568,6 +1568,57 @@ def test_large_march_same_bits_on_any_number_of_ctas(sssp, N, counts):
                 ref = out
 
 
+@pytest.mark.parametrize("N", [16383, 32767, 65535])
+def test_large_march_counts_every_mode_of_the_odd_row(sssp, N):
+    """The stop rule of the large-grid march sums the norms of all modes, also of the row P/2 that one warp of a
+    cluster transforms (modes P/2 + P k2).  Two modes in a constant profile n^2 = 1 + v, so each term stays in its
+    mode: a strong one near the top of the spectrum whose terms fall by 0.04 or less, and in the odd row, at
+    k2 = 16, one whose terms fall by about 0.3 (|b v| < 1, so no mode's terms grow).  A rule that misses the
+    slow mode ends each series after two or three terms instead of six or seven, and the field is 5e-2 off; the
+    bound is the 1e-4 of a field, against FP64."""
+    P = 2 ** ((N + 1).bit_length() // 2)
+    k = np.array([P // 2 + 16 * P, N - 100])
+    H, p, v, tol, steps = 5000.0, 2, -0.1, 1e-3, 2
+    k0 = math.pi * k[0] / (H * math.sqrt(0.05))  # lambda = -0.05 in the slow mode, -3 .. -12 in the other
+    dr = 20.0 / k0
+    lam = -(math.pi * k / (k0 * H)) ** 2
+    b, a, _, _ = sssp.pade_coefficients(k0 * dr, p)
+    n = np.arange(1, N + 1)
+    modes = np.sin(math.pi * np.outer(k, n) / (N + 1))
+    y = np.array([0.5 - 0.2j, 1.0 + 0.3j])
+    u0 = (y @ modes).astype(np.complex64)
+    count = 1  # the final field's transform
+    for _ in range(steps):
+        for bj, aj in zip(b, a):
+            t = w = y / (1.0 + bj * lam)
+            for m in range(1, 12):
+                count += 2
+                t = -bj * v * t / (1.0 + bj * lam)
+                w = w + t
+                if np.sum(np.abs(t) ** 2) <= tol ** 2 * np.sum(np.abs(w) ** 2):
+                    break
+            assert m >= 5
+            y = (aj / bj) * y + (1.0 - aj / bj) * w
+    want = np.exp(1j * k0 * steps * dr) * (y @ modes)
+    ref = None
+    for solves in (1, 39, 77):
+        plans = []
+        for _ in range(solves):
+            pl = sssp.Plan(N, H, k0, dr, p, 12, tol)
+            pl.set_kernel("cta")
+            pl.set_profile(np.full(N, 1.0 + v))
+            pl.set_field(u0)
+            plans.append(pl)
+        sssp.march_batch(plans, steps)
+        u, nd = plans[-1].read_field(), plans[-1].transform_count()
+        for pl in plans:
+            pl.close()
+        assert np.linalg.norm(u - want) / np.linalg.norm(want) <= FIELD_TOL
+        assert nd == count
+        assert ref is None or np.array_equal(u, ref)
+        ref = u
+
+
 # ----------------------------------------------------------------------------- periodic grids of 512 .. 2048 points
 @pytest.mark.parametrize("N", [256, 512, 1024, 2048])
 @pytest.mark.parametrize("terms,absorb", [(1, False), (2, False), (12, False), (5, True)])
