@@ -35,16 +35,18 @@ struct FdCfg {
   static constexpr int WS = NT >= 32 ? 32 : NT;
   static constexpr int NW = (NT + 31) / 32;
   static constexpr unsigned MASK = NT >= 32 ? 0xffffffffu : ((1u << NT) - 1u);
-  // A stage's 48 B of table per point are copied to shared memory a stage ahead (asynchronously, in the
-  // order they lie) into rows of one 16-byte part of one of the thread's points each; the row stride keeps
-  // the copies and the reads on different banks.  Read where they are wanted, a thread's 8 consecutive
+  // Staged form: a stage's 48 B of table per point are copied to shared memory a stage ahead (asynchronously,
+  // in the order they lie) into rows of one 16-byte part of one of the thread's points each; the row stride
+  // keeps the copies and the reads on different banks.  Read where they are wanted, a thread's 8 consecutive
   // points make every load of a warp touch 32 lines, five loads a point: 16 solves of N = 1023, [6/6], 200
-  // steps 4.83 -> 4.06 ms (starters and reads included), the rest the two scans' chains.  Two stages of
-  // L = 4096 do not fit an SM: those tables are read in place.
-  static constexpr bool STAGED = LOG2L <= 11;
+  // steps 4.83 -> 4.06 ms (starters and reads included), the rest the two scans' chains.  Below L = 512 the
+  // copies' address arithmetic and their barrier cost more than the loads they replace, which the L1 serves
+  // (one solve, [8/8], 40 steps, in place / staged: L = 64 305 / 513 us, 128 361 / 517, 256 493 / 542, 512
+  // 753 / 654); two stages of L = 4096 do not fit an SM: those tables are read in place.
+  static constexpr bool STAGEABLE = LOG2L >= 9 && LOG2L <= 11;
   static constexpr int ROW = NT + 1;
   static constexpr int STAGE = 3 * PT * ROW;  // float4 per stage buffer
-  static constexpr size_t SMEM = STAGED ? 2 * sizeof(float4) * STAGE : 0;
+  static constexpr size_t SMEM = 2 * sizeof(float4) * STAGE;  // of the staged form
 };
 
 // affine map x -> a x + b, a and b complex
@@ -98,7 +100,8 @@ __device__ __forceinline__ Aff block_prefix(const Aff& own, Aff* sh) {
   return excl;
 }
 
-template <int LOG2L>
+// STAGED: the tables go through shared memory (the same bits either way)
+template <int LOG2L, bool STAGED>
 __global__ void __launch_bounds__(FdCfg<LOG2L>::NT)
     sssp_fd_march_kernel(const SolveDesc* __restrict__ descs) {
   using C = FdCfg<LOG2L>;
@@ -137,14 +140,14 @@ __global__ void __launch_bounds__(FdCfg<LOG2L>::NT)
   };
   advance(0);
   int buf = 0;
-  if constexpr (C::STAGED) {
+  if constexpr (STAGED) {
     if (d.steps > 0) fetch(0, 0);
   }
   for (int s = 0; s < d.steps; ++s) {
     for (int j = 0; j < d.p; ++j) {
       const FdEntry* gtab = reinterpret_cast<const FdEntry*>(d.fd) + ((size_t)node * d.p + j) * L + P * t;
       const float4* stab = stages + buf * C::STAGE + t;
-      if constexpr (C::STAGED) {
+      if constexpr (STAGED) {
         cp_async_wait<0>();
         __syncthreads();  // everyone's copies of this stage have landed, and the other buffer has been read
         if (j + 1 < d.p) {
@@ -155,9 +158,9 @@ __global__ void __launch_bounds__(FdCfg<LOG2L>::NT)
         }
         buf ^= 1;
       }
-      auto inv = [&](int i) { return C::STAGED ? stab[(3 * i) * C::ROW] : gtab[i].inv; };
-      auto alpha = [&](int i) { return C::STAGED ? stab[(3 * i + 1) * C::ROW] : gtab[i].alpha; };
-      auto mcp = [&](int i) { return C::STAGED ? stab[(3 * i + 2) * C::ROW] : gtab[i].mcp; };
+      auto inv = [&](int i) { return STAGED ? stab[(3 * i) * C::ROW] : gtab[i].inv; };
+      auto alpha = [&](int i) { return STAGED ? stab[(3 * i + 1) * C::ROW] : gtab[i].alpha; };
+      auto mcp = [&](int i) { return STAGED ? stab[(3 * i + 2) * C::ROW] : gtab[i].mcp; };
       // forward sweep g_n = alpha_n g_{n-1} + inv_n y_n
       float2 be[P];
       Aff own{make_float2(1.f, 0.f), make_float2(0.f, 0.f)};
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(FdCfg<LOG2L>::NT)
         y[i] = ffmul(c1, y[i]) + ffmul(c2, w);  // (a_j/b_j) y + (1 - a_j/b_j) w
       }
     }
-    if constexpr (!C::STAGED) advance(s + 1);
+    if constexpr (!STAGED) advance(s + 1);
     const long long gs = d.step0 + s + 1;
     if (d.tl_every > 0 && gs % d.tl_every == 0) {
       const float lr = float(10.0 * log10(d.r0 + double(s + 1) * d.dr));

@@ -3,8 +3,8 @@
 #include <cuda_runtime.h>
 
 #include <complex>
+#include <map>
 #include <mutex>
-#include <set>
 #include <vector>
 
 #include "fd_launch.h"
@@ -14,23 +14,58 @@ namespace sssp_fd {
 
 namespace {
 
+struct Room {
+  int sms = 0, solves = 0;  // SMs of a device, staged solves resident on one
+};
+
+// the staged form's shared-memory attribute and residency on the current device (once a device and size)
 template <int LOG2L>
-cudaError_t launch_t(const sssp::SolveDesc* d, int count, cudaStream_t st) {
+cudaError_t room_for(Room* out) {
   using C = sssp::FdCfg<LOG2L>;
   static std::mutex mu;
-  static std::set<int> done;  // devices whose shared-memory attribute is set
+  static std::map<int, Room> cache;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    if (!done.count(dev)) {
-      e = cudaFuncSetAttribute(sssp::sssp_fd_march_kernel<LOG2L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
-      if (e != cudaSuccess) return e;
-      done.insert(dev);
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = cache.find(dev);
+  if (it == cache.end()) {
+    const auto k = sssp::sssp_fd_march_kernel<LOG2L, true>;
+    Room r;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM))) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.solves, k, C::NT, C::SMEM)) != cudaSuccess) return e;
+    it = cache.emplace(dev, r).first;
+  }
+  *out = it->second;
+  return cudaSuccess;
+}
+
+// Staged tables leave room for S = 4, 2 and 1 solves an SM at L = 512, 1024 and 2048 (read in place: 13, 6 and 3), so
+// more of them march in waves.  With k solves an SM, marches in place take about k times, staged ones about
+// 0.9 S ceil(k / S) times as long as one more solve in place does: L = 1024, [8/8], 40 steps, in place /
+// staged ms: 304 solves 2.11 / 1.66, 400 2.89 / 3.19, 608 3.71 / 3.27, 700 4.48 / 4.84, 912 5.41 / 4.87;
+// L = 512: 608 solves 2.09 / 1.65, 640 2.46 / 2.89, 912 2.93 / 3.06, 1216 3.78 / 3.22; L = 2048 staged at every
+// count (160 solves 3.66 / 3.20, 456 5.32 / 4.91).  One wave gains at every count.
+bool staged(const Room& r, int count) {
+  if (r.sms < 1 || r.solves < 1) return false;
+  const int k = (count + r.sms - 1) / r.sms, waves = (k + r.solves - 1) / r.solves;
+  return waves == 1 || 9LL * r.solves * waves <= 10LL * k;
+}
+
+template <int LOG2L>
+cudaError_t launch_t(const sssp::SolveDesc* d, int count, cudaStream_t st) {
+  using C = sssp::FdCfg<LOG2L>;
+  if constexpr (C::STAGEABLE) {
+    Room r;
+    const cudaError_t e = room_for<LOG2L>(&r);
+    if (e != cudaSuccess) return e;
+    if (staged(r, count)) {
+      sssp::sssp_fd_march_kernel<LOG2L, true><<<count, C::NT, C::SMEM, st>>>(d);
+      return cudaGetLastError();
     }
   }
-  sssp::sssp_fd_march_kernel<LOG2L><<<count, C::NT, C::SMEM, st>>>(d);
+  sssp::sssp_fd_march_kernel<LOG2L, false><<<count, C::NT, 0, st>>>(d);
   return cudaGetLastError();
 }
 

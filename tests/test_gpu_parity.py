@@ -6,6 +6,7 @@ FP32 rounding bound of a length-L FFT (a few 1e-6 relative).
 """
 import math
 import os
+import time
 
 import numpy as np
 import pytest
@@ -1662,3 +1663,42 @@ def test_fdssp_staged_tables_against_oracle(sssp, N, p):
     tl, _ = pl.read_tl()
     pl.close()
     _compare(u, tl, _fd_oracle(s, 3))
+
+
+@pytest.mark.parametrize("N,count", [(511, 640), (1023, 320), (255, 3)])
+def test_fdssp_tables_staged_or_in_place_same_bits(sssp, N, count):
+    """One solve and a batch of the same solve just beyond what the staged form holds at once (where
+    the tables are read in place): the same bits, field and TL rows."""
+    s = inputs.munk(N=N, freq=0.02 * (N + 1), dr=50.0, steps=3, pade_order=3)
+    out = []
+    for n in (1, count):
+        plans = [sssp.plan_for(s, tl_every=1, op="fd3") for _ in range(n)]
+        sssp.march_batch(plans, s.steps)
+        out.append((plans[-1].read_field(), plans[-1].read_tl()[0]))
+        for pl in plans:
+            pl.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("small,large,most", [((63, 1), (255, 1), 0.8), ((511, 640), (511, 1216), 0.8)])
+def test_fdssp_time_grows_with_the_work(sssp, small, large, most):
+    """The FD-SSP march takes less time for a quarter of the points, and for half the solves: 0.62 and 0.71 of
+    the other's time with the tables read in place, 0.95 and 0.89 where they are staged at any size and count."""
+    import torch
+    times = []
+    for N, count in (small, large):
+        s = inputs.munk(N=N, freq=0.02 * (N + 1) + 1.0, dr=25.0, steps=60, pade_order=8)
+        plans = [sssp.plan_for(s, op="fd3") for _ in range(count)]
+        best = math.inf
+        for _ in range(6):
+            for pl in plans:
+                pl.set_field(s.u0)
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            sssp.march_batch(plans, s.steps)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        for pl in plans:
+            pl.close()
+        times.append(best)
+    assert times[0] <= most * times[1], times
