@@ -107,7 +107,8 @@ pe_status pe_set_output(pe_plan* plan, int tl_every);
 /*
  * Set the field u(r, z_n), n = 1..N, at range r [m] (the starter, Section 3.2).
  *   u          N interleaved complex64 values (2N floats)
- *   on_device  0: u is host memory (copied before return); 1: u is device memory
+ *   on_device  0: u is host memory (copied before return); 1: u is device memory (read where it lies on
+ *              the plan's device, copied from another device's or pinned host memory)
  * Resets the step counter and the recorded TL rows.  Errors: PE_ERR_ARG (NULL u),
  * PE_ERR_CUDA.
  */

@@ -21,6 +21,7 @@
 #include "eo_launch.h"
 #include "march_kernel.cuh"
 #include "march_large.cuh"
+#include "memory_reach.h"
 #include "fd_launch.h"
 #include "pade_host.h"
 #include "plan_internal.h"
@@ -813,9 +814,9 @@ pe_status pe_set_field(pe_plan* p, const float* u, int on_device, double r) {
   NvtxRange nvtx_("pe_set_field");
   if (!u) return fail(p, PE_ERR_ARG, "u is NULL");
   if (!std::isfinite(r)) return fail(p, PE_ERR_ARG, "r must be finite");
-  // a device field is read where it lies (complex values at an 8-byte boundary), others are staged
+  // a field on the plan's device is read where it lies (complex values at an 8-byte boundary), others are staged
   const float2* src = reinterpret_cast<const float2*>(u);
-  if (!on_device || reinterpret_cast<uintptr_t>(u) % sizeof(float2) != 0) {
+  if (!on_device || reinterpret_cast<uintptr_t>(u) % sizeof(float2) != 0 || !sssp::reached_in_place(u, p->device)) {
     PE_CUDA(p, cudaMemcpyAsync(p->dStage, u, sizeof(float2) * p->N_user,
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, p->stream));
     src = p->dStage;
@@ -1226,10 +1227,10 @@ pe_status pe_dst1_batch(pe_plan* p, const float* in, float* out, int count) {
   const uintptr_t ia = reinterpret_cast<uintptr_t>(in), oa = reinterpret_cast<uintptr_t>(out);
   const size_t bytes = sizeof(float2) * size_t(p->N) * size_t(count);
   // The L >= 512 kernels write the packed rows themselves (every field is read before it is written, so
-  // in place too).  Elsewhere -- and for result addresses or overlaps that need the detour -- a field gets
-  // an L-long result row (index 0 is the zero mode), then rows 1..N are packed.
+  // in place too).  Elsewhere -- and for result addresses, memory or overlaps that need the detour -- a field
+  // gets an L-long result row (index 0 is the zero mode), then rows 1..N are packed.
   const bool direct = p->bc == PE_BC_DIRICHLET && p->log2L >= sssp_eo::kMinLog2 && oa % sizeof(float2) == 0 &&
-                      (ia == oa || ia + bytes <= oa || oa + bytes <= ia);
+                      (ia == oa || ia + bytes <= oa || oa + bytes <= ia) && sssp::reached_in_place(out, p->device);
   float2* res = nullptr;
   float2* work = nullptr;
   if (!direct)

@@ -220,3 +220,26 @@ def test_shape_entry_points_reject_null_plans(L):
     assert lib.pe_march_batch_autotune(None, 1, 4, None, None, None) == sssp.PE_ERR_ARG
     assert sssp.SHAPE_NAMES[3:] == ("cluster8_pull", "cluster8_push", "cluster16_pull", "cluster16_push")
     assert len(sssp.SHAPE_NAMES) == 7  # PE_AUTOTUNE_SHAPES in include/sssp.h
+
+
+def test_which_memory_the_kernels_use_in_place(L, tmp_path):
+    """A caller's array is read and written where it lies only in the plan's own device's memory or managed
+    memory; another device's, pinned and unregistered host memory take the copy they took before."""
+    import subprocess
+    from paper_2511_03343_gb300 import build
+    src = tmp_path / "reach.cpp"
+    src.write_text("""#include "memory_reach.h"
+#include <cstdio>
+#include <initializer_list>
+int main() {
+  for (cudaMemoryType t : {cudaMemoryTypeUnregistered, cudaMemoryTypeHost, cudaMemoryTypeDevice, cudaMemoryTypeManaged})
+    for (int owner = 0; owner < 2; ++owner) std::printf("%d", int(sssp::reached_in_place(t, owner, 1)));
+}
+""")
+    subprocess.run([build._nvcc(), "-std=c++17", "-I", build.CSRC, str(src), "-o", str(tmp_path / "reach")], check=True)
+    got = subprocess.run([str(tmp_path / "reach")], check=True, capture_output=True, text=True).stdout
+    assert got == "00" "00" "01" "11"
+    abi = open(os.path.join(build.CSRC, "sssp_abi.cu")).read()
+    for entry, arg in (("pe_set_field", "u"), ("pe_dst1_batch", "out")):
+        body = abi[abi.index(f"pe_status {entry}("):]
+        assert f"reached_in_place({arg}, p->device)" in body[:body.index("\n}\n")]

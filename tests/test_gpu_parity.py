@@ -1702,3 +1702,26 @@ def test_fdssp_time_grows_with_the_work(sssp, small, large, most):
             pl.close()
         times.append(best)
     assert times[0] <= most * times[1], times
+
+
+@pytest.mark.parametrize("N", [255, 511, 4095, 8191])
+def test_pinned_host_arrays_given_as_device_memory(sssp, N):
+    """Pinned host memory passed where device memory is meant is copied, as a starter and as the batched
+    transform's result: the same bits as through device memory."""
+    import torch
+    g = torch.Generator().manual_seed(N)
+    x = torch.randn(3, N, generator=g, dtype=torch.complex64)
+    dev, host = x.cuda(), x.pin_memory()
+    pl = sssp.Plan(N, 100.0, 0.4, 5.0, 4)
+    states = []
+    for u in (dev, host):
+        pl._c(sssp.lib().pe_set_field(pl.handle, u.data_ptr(), 1, 0.0))
+        assert np.array_equal(pl.read_field(), x[0].numpy())
+        states.append(pl.save_state()[0])
+    assert np.array_equal(states[0], states[1])
+    want, got = torch.empty_like(dev), torch.empty_like(x).pin_memory()
+    pl.dst1_batch(dev, want)
+    pl._c(sssp.lib().pe_dst1_batch(pl.handle, dev.data_ptr(), got.data_ptr(), 3))
+    pl.sync()
+    pl.close()
+    assert torch.equal(torch.view_as_real(got), torch.view_as_real(want.cpu()))
