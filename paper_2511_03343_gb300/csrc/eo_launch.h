@@ -15,8 +15,8 @@ constexpr int kMinLog2 = 9;        // the transform
 constexpr int kMinMarchLog2 = 11;  // the march
 constexpr int kMaxLog2 = 12;
 
-inline bool supported(int log2L) { return log2L >= kMinLog2 && log2L <= kMaxLog2; }
-inline bool march_supported(int log2L) { return log2L >= kMinMarchLog2 && log2L <= kMaxLog2; }
+constexpr bool supported(int log2L) { return log2L >= kMinLog2 && log2L <= kMaxLog2; }
+constexpr bool march_supported(int log2L) { return log2L >= kMinMarchLog2 && log2L <= kMaxLog2; }
 // build the current device's tables of a size (kept for the process; plan creation calls it so that a
 // march allocates nothing)
 cudaError_t prepare(int log2L);

@@ -160,7 +160,7 @@ cudaError_t set_smem_attr() {
   const int sm = int(Cfg<LOG2L>::SMEM), smc = int(Cfg<LOG2L>::SMEM_CPLX);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic>, a, sm);
-  if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
+  if constexpr (!sssp_eo::march_supported(LOG2L)) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet>, a, sm);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet>, a, smc);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet>, a, sm);
@@ -186,8 +186,9 @@ cudaError_t launch_march_t(const SolveDesc* dDescs, int count, const TransformTa
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcPeriodic><<<dim3(count, split), nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
       sssp::sssp_march_kernel<LOG2L, false, sssp::kBcPeriodic><<<dim3(count, split), nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
-  } else if constexpr (LOG2L < sssp_eo::kMinMarchLog2) {
-    if (cplx)
+  } else {
+    if constexpr (sssp_eo::march_supported(LOG2L)) return cudaErrorInvalidValue;  // likewise
+    else if (cplx)
       sssp::sssp_march_kernel<LOG2L, true, sssp::kBcDirichlet><<<dim3(count, split), nt, smc, st>>>(dDescs, tabs.tw, tabs.sinw);
     else
       sssp::sssp_march_kernel<LOG2L, false, sssp::kBcDirichlet><<<dim3(count, split), nt, sm, st>>>(dDescs, tabs.tw, tabs.sinw);
@@ -201,12 +202,15 @@ cudaError_t launch_dst_t(const float2* in, float2* out, float scale, const Trans
                          const sssp::StartArgs& sa = {}) {
   cudaError_t e = set_smem_attr<LOG2L>();
   if (e != cudaSuccess) return e;
-  if (bc == sssp::kBcPeriodic)
+  if (bc == sssp::kBcPeriodic) {
     sssp::sssp_dst_kernel<LOG2L, sssp::kBcPeriodic><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM0, st>>>(
         in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
-  else if constexpr (LOG2L < sssp_eo::kMinMarchLog2)
-    sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM0, st>>>(
-        in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
+  } else {
+    if constexpr (sssp_eo::march_supported(LOG2L)) return cudaErrorInvalidValue;  // the caller's other branch
+    else
+      sssp::sssp_dst_kernel<LOG2L, sssp::kBcDirichlet><<<count, Cfg<LOG2L>::NT, Cfg<LOG2L>::SMEM0, st>>>(
+          in, out, scale, tabs.tw, tabs.sinw, in_stride, out_stride, sa);
+  }
   return cudaGetLastError();
 }
 
@@ -373,6 +377,7 @@ cudaError_t launch_dst(int log2L, const float2* in, float2* out, float scale, co
                        int off = 1, const sssp::StartArgs& sa = {}) {
   if (bc == sssp::kBcDirichlet && (sa.status ? sssp_eo::march_supported(log2L) : sssp_eo::supported(log2L)))
     return sssp_eo::launch_dst(log2L, in, out, scale, count, is, os, off, st, sa);
+  if (log2L <= kMaxSmemLog2 && off != 1) return cudaErrorInvalidValue;  // the scan form writes mode 0 too
   switch (log2L) {
     case 3: return launch_dst_t<3>(in, out, scale, tabs, st, count, is, os, bc, sa);
     case 4: return launch_dst_t<4>(in, out, scale, tabs, st, count, is, os, bc, sa);
