@@ -82,7 +82,11 @@ struct BigCfg {
   static constexpr size_t SMEM = sizeof(float2) * 2 * size_t(BUF) + sizeof(float4) * (P + Q + R + NT1 + Q / 2);
   // the march also holds the two buffers of a one-warp FFT (the column Q/2 or the row P/2)
   static constexpr size_t SMEM_MARCH = SMEM + sizeof(float2) * 2 * (RSP > RSQ ? RSP : RSQ);
-  static constexpr int CTAS = NA - 1;  // CTAs of a march's cluster: a tile of each pass each
+  static constexpr int CTAS = NA - 1;  // CTAs of a march's cluster, at most: a tile of each pass each
+  // the norm partials of the stop test are summed over GT tiles at a time, the share of a CTA of the largest
+  // cluster launched (4), so that the sums are the same on any number of CTAs (77 solves of N = 65535, 3 steps:
+  // a sum per tile 55.4 ms, per GT tiles 55.1)
+  static constexpr int GT = CTAS > 4 ? CTAS / 4 : 1, SLOTS = CTAS / GT;
   static_assert(NA == NBT, "as many tiles in either pass");
 };
 
@@ -535,6 +539,7 @@ struct SnkArr {
 };
 // The partial sum w_j = t_0 + t_1 + .. is kept itself (not t_1 + .. beside t_0), so a term
 // streams B and w, and the stage's combine reads t_0 once: y <- R y + beta (w - t_0).
+template <int CTAS, int GT>
 struct SnkTerm {  // t_m = B_k S_k: w += t_m, X = t_m, and the norm partials of the stop test
   static constexpr bool kL2 = true;
   __device__ __forceinline__ void l2(int k) {
@@ -544,16 +549,17 @@ struct SnkTerm {  // t_m = B_k S_k: w += t_m, X = t_m, and the norm partials of 
   const float2* B;
   float2* w;
   float2* X;
-  float2* red;  // shared memory: the norm partials of tile i and warp v at i NW + v
+  float2* red;  // shared memory: the norm partials of tiles GT i .. GT i + GT - 1 and warp v at i NW + v
   float nt, nw;
   float2 pb[kLargePT / 2], pw[kLargePT / 2];  // B and w of the tile's outputs
+  // Both sums in one chain of shuffles: after the first step the lower half-warp carries nt, the upper nw.
   __device__ __forceinline__ void tile_end(int i) {
+    if (i < CTAS && i % GT != GT - 1) return;
+    const bool up = threadIdx.x & 16;
+    float v = (up ? nw : nt) + __shfl_xor_sync(0xffffffffu, up ? nt : nw, 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      nt += __shfl_xor_sync(0xffffffffu, nt, o);
-      nw += __shfl_xor_sync(0xffffffffu, nw, o);
-    }
-    if ((threadIdx.x & 31) == 0) red[i * (kLargeNT / 32) + (threadIdx.x >> 5)] = make_float2(nt, nw);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 15) == 0) reinterpret_cast<float*>(red)[i / GT * (kLargeNT / 16) + (threadIdx.x >> 4)] = v;
     nt = nw = 0.f;
   }
   // The odd row's partials, lane i < G holding the outputs i + G q.  A tile of TR rows gives these to the
@@ -566,7 +572,7 @@ struct SnkTerm {  // t_m = B_k S_k: w += t_m, X = t_m, and the norm partials of 
       nt += __shfl_xor_sync(0xffffffffu, nt, 1);
       nw += __shfl_xor_sync(0xffffffffu, nw, 1);
     }
-    if (lane % PER == 0 && lane / PER < kLargeNT / 32) red[i * (kLargeNT / 32) + lane / PER] = make_float2(nt, nw);
+    if (lane % PER == 0 && lane / PER < kLargeNT / 32) red[i / GT * (kLargeNT / 32) + lane / PER] = make_float2(nt, nw);
     nt = nw = 0.f;
   }
   __device__ __forceinline__ void prefetch(int q, int k) {
@@ -609,9 +615,9 @@ __global__ void __launch_bounds__(kLargeNT, 1)
   constexpr int L = C::L;
   extern __shared__ __align__(16) float2 tile_smem[];
   __shared__ SolveDesc d;
-  constexpr int TILES = BigCfg<LOG2L>::CTAS, T = TILES / NC;  // tiles of a pass, and of this CTA
-  __shared__ float2 red[(TILES + 1) * C::NW];                 // norm partials of the stop test: per tile and warp,
-  __shared__ float2 part[TILES + 1];                          // per tile and for the odd row (every CTA's)
+  using B = BigCfg<LOG2L>;
+  __shared__ float2 red[(B::SLOTS + 1) * C::NW];  // norm partials of the stop test: per GT tiles and warp,
+  __shared__ float2 part[B::SLOTS + 1];           // per GT tiles and for the odd row (every CTA's)
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   const int t = threadIdx.x, rank = int(cl.block_rank());
   {
@@ -665,12 +671,12 @@ __global__ void __launch_bounds__(kLargeNT, 1)
         ++ndst;
         float first = 0.f;
         for (int m = 1; m < d.terms; ++m) {
-          SnkTerm sk{d.B + (size_t)j * L, wsum, X, red, 0.f, 0.f, {}, {}};
+          SnkTerm<B::CTAS, B::GT> sk{d.B + (size_t)j * L, wsum, X, red, 0.f, 0.f, {}, {}};
           dst_cluster<LOG2L, NC>(W, tile_smem, SrcV{X, V, Vi}, sk, rank);  // B DST(V t_{m-1}), w += t_m
           ++ndst;
-          // (pass B ends with a block barrier) the totals of this CTA's tiles, to every CTA: summed per tile
-          // and then in tile order, so that the decision does not depend on the tiles' split over CTAs
-          constexpr int MINE = NC == 1 ? TILES + 1 : T;  // one CTA: its last tile is the odd row
+          // (pass B ends with a block barrier) the totals of this CTA's tiles, to every CTA: summed per GT tiles
+          // and then in their order, so that the decision does not depend on the tiles' split over CTAs
+          constexpr int MINE = NC == 1 ? B::SLOTS + 1 : B::SLOTS / NC;  // one CTA: its last tile is the odd row
           auto total = [&](int c) {
             float2 v = make_float2(0.f, 0.f);
 #pragma unroll
@@ -681,13 +687,13 @@ __global__ void __launch_bounds__(kLargeNT, 1)
             if (t < MINE) part[t] = total(t);
           } else {
             if (t < MINE * NC) cl.map_shared_rank(part, t / MINE)[rank * MINE + t % MINE] = total(t % MINE);
-            if (rank == NC - 1 && t >= kLargeNT - NC) cl.map_shared_rank(part, kLargeNT - 1 - t)[TILES] = total(TILES);
+            if (rank == NC - 1 && t >= kLargeNT - NC) cl.map_shared_rank(part, kLargeNT - 1 - t)[B::SLOTS] = total(B::SLOTS);
           }
           solve_sync<NC>();  // the term's results and every CTA's partials
           if (m == d.terms - 1) break;
           float snt = 0.f, snw = 0.f;
 #pragma unroll
-          for (int c = 0; c <= TILES; ++c) {  // the same order in every CTA: a uniform decision
+          for (int c = 0; c <= B::SLOTS; ++c) {  // the same order in every CTA: a uniform decision
             snt += part[c].x;
             snw += part[c].y;
           }
