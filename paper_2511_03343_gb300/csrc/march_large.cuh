@@ -30,7 +30,6 @@ struct CfgL {
   static constexpr int L = 1 << LOG2L;
   static constexpr int NT = kLargeNT;
   static constexpr int NW = NT / 32;
-  static constexpr int PER = L / NT;        // elements per thread in element-wise loops
 };
 
 // A hint that moves the 128-byte line holding p into the L2 (no registers held; p is always an

@@ -278,36 +278,66 @@ cudaError_t large_tabs(sssp::LargeTabs* out) {
 constexpr int kLargeTileFields = 32;
 
 template <int LOG2L, int CTAS>
-cudaError_t launch_march_large_n(const SolveDesc* dDescs, int count, const sssp::LargeTabs& tb, cudaStream_t st) {
-  constexpr int NC = kLargeCtas<LOG2L, CTAS>;
-  cudaLaunchConfig_t cfg{};
+struct LargeLaunch {
+  static constexpr int NC = kLargeCtas<LOG2L, CTAS>;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = NC;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(unsigned(NC) * unsigned(count));
-  cfg.blockDim = dim3(sssp::kLargeNT);
-  // one CTA needs no buffers for the odd column and row: 8.7 KB less at L = 65536, where the SM then keeps 32 KB
-  // more of L1 (152 solves, N = 65535, 3 steps, [6/6]: 59.4 -> 58.8 ms)
-  cfg.dynamicSmemBytes = NC == 1 ? sssp::BigCfg<LOG2L>::SMEM : sssp::BigCfg<LOG2L>::SMEM_MARCH;
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, sssp::sssp_march_large_kernel<LOG2L, NC>, dDescs, tb);
+  cudaLaunchConfig_t cfg{};
+  LargeLaunch(int count, cudaStream_t st) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = NC;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(unsigned(NC) * unsigned(count));
+    cfg.blockDim = dim3(sssp::kLargeNT);
+    // one CTA needs no buffers for the odd column and row: 8.7 KB less at L = 65536, where the SM then keeps 32 KB
+    // more of L1 (152 solves, N = 65535, 3 steps, [6/6]: 59.4 -> 58.8 ms)
+    cfg.dynamicSmemBytes = NC == 1 ? sssp::BigCfg<LOG2L>::SMEM : sssp::BigCfg<LOG2L>::SMEM_MARCH;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  cudaError_t march(const SolveDesc* d, const sssp::LargeTabs& tb) {
+    return cudaLaunchKernelEx(&cfg, sssp::sssp_march_large_kernel<LOG2L, NC>, d, tb);
+  }
+};
+
+// solves of CTAS CTAs that the current device runs at once (after large_tabs has set the kernels' attributes)
+template <int LOG2L, int CTAS>
+cudaError_t large_room(int* solves) {
+  static std::mutex mu;
+  static std::map<int, int> cache;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = cache.find(dev);
+  if (it == cache.end()) {
+    LargeLaunch<LOG2L, CTAS> one(1, nullptr);
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, sssp::sssp_march_large_kernel<LOG2L, LargeLaunch<LOG2L, CTAS>::NC>, &one.cfg);
+    if (e != cudaSuccess) return e;
+    it = cache.emplace(dev, n).first;
+  }
+  *solves = it->second;
+  return cudaSuccess;
 }
 
-// As many CTAs a solve as the 152 SMs hold at once, up to 4 (the results do not depend on it).  N = 65535,
-// 2 steps, against one CTA a solve: 1 solve 14.0 -> 4.7 ms, 38 solves 15.0 -> 10.3, 76 solves 15.3 -> 11.2 (two CTAs
-// each); with 152 solves one CTA each takes 17.8, two or four 28 (an SM does a tile as fast, the barriers
-// and the single tiles' unhidden loads come on top).  N = 32767 1 solve 7.0 -> 2.3, N = 16383 8.2 -> 4.5 ms.
+// As many CTAs a solve as the device holds of all solves at once, up to 4 (the results do not depend on it).
+// Clusters of 4 need their SMs within a GPC, so the 152 SMs hold 36 of them, not 38.  N = 65535, 3 steps, [6/6],
+// against one CTA a solve: 1 solve 51 -> 17 ms, 36 solves 53 -> 20.3, 37 solves 53 -> 34.9 (two CTAs each; four in two
+// waves 37.8), 76 solves 54.5 -> 40.4; with 152 solves one CTA each takes 58.5, and two or four took 1.6 times as
+// long (an SM does a tile as fast, the barriers and the single tiles' unhidden loads come on top).
+// N = 32767 1 solve 25.6 -> 8.2, N = 16383 (two CTAs at most) 14.6 -> 7.9 ms.
 template <int LOG2L>
 cudaError_t launch_march_large_t(const SolveDesc* dDescs, int count, const TransformTables&, cudaStream_t st) {
   sssp::LargeTabs tb;
+  int four = 0, two = 0;
   cudaError_t e = large_tabs<LOG2L>(&tb);
+  if (e == cudaSuccess) e = large_room<LOG2L, 4>(&four);
+  if (e == cudaSuccess) e = large_room<LOG2L, 2>(&two);
   if (e != cudaSuccess) return e;
-  if (count <= 38) return launch_march_large_n<LOG2L, 4>(dDescs, count, tb, st);
-  if (count <= 76) return launch_march_large_n<LOG2L, 2>(dDescs, count, tb, st);
-  return launch_march_large_n<LOG2L, 1>(dDescs, count, tb, st);
+  if (count <= four) return LargeLaunch<LOG2L, 4>(count, st).march(dDescs, tb);
+  if (count <= two) return LargeLaunch<LOG2L, 2>(count, st).march(dDescs, tb);
+  return LargeLaunch<LOG2L, 1>(count, st).march(dDescs, tb);
 }
 
 template <int LOG2L>
@@ -335,8 +365,14 @@ cudaError_t launch_dst_large_t(const float2* in, float2* out, float scale, float
 // 48 us on 100 (march call to completion).
 cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const TransformTables& tabs, cudaStream_t st,
                          bool cplx, int bc, int ppt, int iso_rows) {
-  constexpr int kRoom = 304;  // two CTAs on each of the 152 SMs
-  const int split = std::max(1, std::min(iso_rows, kRoom / count));
+  int split = 1;
+  if (iso_rows > 1) {  // two CTAs on each SM
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    split = std::max(1, std::min(iso_rows, 2 * sms / count));
+  }
   if (ppt != 8) {  // the one-CTA kernel at 4 or 16 points per thread (Dirichlet, L <= 4096)
     if (bc != sssp::kBcDirichlet) return cudaErrorInvalidValue;
     return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx, split);

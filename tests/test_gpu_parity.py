@@ -1725,3 +1725,26 @@ def test_pinned_host_arrays_given_as_device_memory(sssp, N):
     pl.sync()
     pl.close()
     assert torch.equal(torch.view_as_real(got), torch.view_as_real(want.cpu()))
+
+
+def test_large_march_solves_that_run_at_once(sssp):
+    """Where a device holds so many solves of N = 65535 on clusters of 4 CTAs, one solve more runs on clusters of 2
+    and not in a second wave: no count up to 39 takes longer than 39 solves do (37 in two waves: 1.08 times)."""
+    import torch
+    s = inputs.munk(N=65535, freq=300.0, dr=25.0, steps=1, pade_order=2)
+    plans = [sssp.plan_for(s) for _ in range(39)]
+    took = {}
+    for count in range(35, 40):
+        best = math.inf
+        for _ in range(4):
+            for pl in plans[:count]:
+                pl.set_field(s.u0)
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            sssp.march_batch(plans[:count], 1)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        took[count] = best
+    for pl in plans:
+        pl.close()
+    assert max(took.values()) <= 1.04 * took[39], took
