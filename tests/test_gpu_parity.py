@@ -1748,3 +1748,40 @@ def test_large_march_solves_that_run_at_once(sssp):
     for pl in plans:
         pl.close()
     assert max(took.values()) <= 1.04 * took[39], took
+
+
+@pytest.mark.parametrize("N,bc", [(255, "dirichlet"), (511, "dirichlet"), (1023, "dirichlet"), (2047, "dirichlet"), (4095, "dirichlet"),
+                                  (256, "periodic"), (512, "periodic"), (2048, "periodic"), (1025, "neumann"),
+                                  (16383, "dirichlet"), (65535, "dirichlet")])
+def test_diverged_and_non_finite_series_end_every_one_cta_kernel(sssp, N, bc):
+    """The exits of the stop rule in each kernel of PE_KERNEL_CTA, in a batch beside a solve that converges: a profile
+    far outside the series' convergence region reports PE_ERR_NEUMANN_DIVERGED, a field whose squares overflow
+    PE_ERR_NUMERIC, each march of a plan again, and the other solve and the plan's next field are untouched."""
+    u = np.exp(-((np.arange(N) / N - 0.4) / 0.1) ** 2).astype(np.complex64)
+
+    def plan(n2):
+        pl = sssp.Plan(N, 100.0, 0.4, 5.0, 4, 12, 1e-10, bc=bc)
+        if bc == "dirichlet":
+            pl.set_kernel("cta")
+        pl.set_profile(np.full(N, n2), 0.0)
+        pl.set_field(u)
+        return pl
+
+    good, far, big = plan(1.01), plan(40.0), plan(1.01)
+    good.march(3)
+    want = good.read_field()
+    for _ in range(2):
+        good.set_field(u)
+        far.set_field(u)
+        big.set_field(np.full(N, 3e30, dtype=np.complex64))
+        sssp.march_batch([far, good, big], 3)
+        for pl, status in ((far, sssp.PE_ERR_NEUMANN_DIVERGED), (big, sssp.PE_ERR_NUMERIC)):
+            with pytest.raises(sssp.PEError) as e:
+                pl.sync()
+            assert e.value.status == status
+        assert np.array_equal(good.read_field(), want)
+    big.set_field(u)
+    big.march(3)
+    assert np.array_equal(big.read_field(), want)
+    for pl in (good, far, big):
+        pl.close()
