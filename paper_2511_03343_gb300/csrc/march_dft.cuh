@@ -44,11 +44,19 @@ struct DThread {
   }
 };
 
-// twiddles kept in registers: w_M^{c k1}; w_Q^{v s} of the H-point sub-rows (v = h + H vv); w_{8Q}^{m2 k2}, k2 = h + H w
+// twiddles kept in registers: w_M^{c k1}; w_Q^{v s} of the H-point sub-rows (v = h + H vv), hi + lo; w_{8Q}^{m2 k2},
+// k2 = h + H w.  wM: the M FP32 roots, then the lo parts of w_Q^j, j < Q.
+// The sub-rows' lo parts: a twiddle's FP32 representation error is the same in every transform and adds up over
+// the steps, and the extra pass over H points gave these transforms more of it than the general passes have.
+// Field error against complex128, 40 steps, [6/6], mean of 128 solves, general passes / all FP32 / sub-rows hi +
+// lo: 1024 points 6.35e-7 / 6.60e-7 / 6.11e-7, 2048 7.85e-7 / 8.95e-7 / 6.70e-7.  March of 30 steps: 1024 points 1.73 ->
+// 1.78 ms, 2048 points 2.98 -> 2.86 ms (the general passes: 2.25 and 4.48).  hi + lo in the third pass too gives 6.0e-7
+// and 6.5e-7, but 2.11 ms at 1024 points (registers spill).
 template <int LOG2M>
 struct DTw {
   static constexpr int Q = DCfg<LOG2M>::Q, H = DCfg<LOG2M>::H;
-  float2 a[7], b[H > 1 ? 8 : 1], m[8];
+  float2 a[7], m[8];
+  float4 b[H > 1 ? 8 : 1];
   __device__ __forceinline__ void load(const float2* wM, const DThread<LOG2M>& th) {
 #pragma unroll
     for (int k = 1; k < 8; ++k) a[k - 1] = __ldg(wM + th.c * k);
@@ -58,7 +66,11 @@ struct DTw {
 #pragma unroll
       for (int vv = 0; vv < 8 / H; ++vv)
 #pragma unroll
-        for (int s = 0; s < H; ++s) b[vv * H + s] = __ldg(wM + 64 * (th.h + H * vv) * s);
+        for (int s = 0; s < H; ++s) {
+          const int j = (th.h + H * vv) * s;  // below 8 H = Q
+          const float2 hi = __ldg(wM + 64 * j), lo = __ldg(wM + DCfg<LOG2M>::M + j);
+          b[vv * H + s] = make_float4(hi.x, hi.y, lo.x, lo.y);
+        }
     }
   }
 };
@@ -91,7 +103,7 @@ __device__ __forceinline__ void dft_regs(float2 (&a)[8], const DTw<LOG2M>& tw, c
       if constexpr (H == 2) dft2(b[0], b[1]);
       else dft4(b[0], b[1], b[2], b[3]);
 #pragma unroll
-      for (int q = 0; q < H; ++q) A[(q * 8 + th.m2) * K::SP + v] = q ? cmul(b[q], tw.b[vv * H + q]) : b[0];
+      for (int q = 0; q < H; ++q) A[(q * 8 + th.m2) * K::SP + v] = q ? ffmul(tw.b[vv * H + q], b[q]) : b[0];
     }
     __syncwarp();
 #pragma unroll
@@ -118,8 +130,8 @@ __device__ __forceinline__ float2 ldv2(const float2* p) {
   return v;
 }
 
-// The march: blockIdx.x selects the solve.  (2048 points: 3040 -> 2040 cycles a transform at 2.07 GHz for one
-// solve, the general kernel against this one; 24 rigid-boundary solves of N = 1025, 60 steps, 11.9 -> 7.8 ms.)
+// The march: blockIdx.x selects the solve.  (2048 points, one solve, 30 steps, the general kernel
+// against this one: 4.48 -> 2.86 ms; 152 solves 5.46 -> 3.33, 304 9.29 -> 6.46.)
 template <int LOG2M, bool CPLX>
 __global__ void __launch_bounds__(DCfg<LOG2M>::NT, DCfg<LOG2M>::MIN_BLOCKS)
     sssp_march_dft_kernel(const SolveDesc* __restrict__ descs, const float2* __restrict__ wM) {

@@ -15,7 +15,7 @@ namespace sssp_dft {
 namespace {
 
 std::mutex g_mu;
-std::map<std::pair<int, int>, const float2*> g_tabs;  // (device, log2M): e^{-2 pi i e/M}, e in [0, M)
+std::map<std::pair<int, int>, const float2*> g_tabs;  // (device, log2M): the roots of DTw
 
 template <int LOG2M>
 cudaError_t set_attrs() {
@@ -37,12 +37,14 @@ cudaError_t tabs_for(int log2M, const float2** out) {
   }
   e = log2M == 9 ? set_attrs<9>() : (log2M == 10 ? set_attrs<10>() : set_attrs<11>());
   if (e != cudaSuccess) return e;
-  const int M = 1 << log2M;
-  std::vector<float2> h(M);
+  const int M = 1 << log2M, Q = M / 64;
+  std::vector<float2> h(M + Q);
   for (int i = 0; i < M; ++i) h[i] = make_float2(float(std::cos(2.0 * M_PI * i / M)), float(-std::sin(2.0 * M_PI * i / M)));
+  for (int j = 0; j < Q; ++j)
+    h[M + j] = make_float2(float(std::cos(2.0 * M_PI * j / Q) - double(h[64 * j].x)), float(-std::sin(2.0 * M_PI * j / Q) - double(h[64 * j].y)));
   float2* d = nullptr;
-  if ((e = cudaMalloc(&d, sizeof(float2) * M)) != cudaSuccess) return e;
-  if ((e = cudaMemcpy(d, h.data(), sizeof(float2) * M, cudaMemcpyHostToDevice)) != cudaSuccess) {
+  if ((e = cudaMalloc(&d, sizeof(float2) * h.size())) != cudaSuccess) return e;
+  if ((e = cudaMemcpy(d, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
     cudaFree(d);
     return e;
   }

@@ -1785,3 +1785,23 @@ def test_diverged_and_non_finite_series_end_every_one_cta_kernel(sssp, N, bc):
     assert np.array_equal(big.read_field(), want)
     for pl in (good, far, big):
         pl.close()
+
+
+def test_periodic_march_rounding(sssp):
+    """The periodic march of 2048 points rounds no more than the general passes do: 40 steps from a field of random
+    propagating modes, six frequencies; mean field error against FP64 over such solves 7.85e-7 with the general
+    passes, 8.95e-7 with every twiddle of the register passes one FP32 number, 6.7e-7 with the sub-rows' as hi + lo."""
+    N, steps, err = 2048, 40, []
+    for i, f in enumerate(np.linspace(154.0, 307.0, 6)):
+        s = inputs.munk(N=N, freq=f, dr=25.0, steps=steps, pade_order=6, bc="periodic")
+        rng = np.random.default_rng(i)
+        M = int(0.5 * s.k0 * s.H / math.pi)
+        a = (rng.standard_normal(M) + 1j * rng.standard_normal(M)) / math.sqrt(M)
+        X = np.zeros(N, dtype=complex)
+        X[1:M // 2 + 1] = a[:M // 2]
+        X[N - (M - M // 2):] = a[M // 2:]
+        s.u0 = (np.fft.ifft(X) * N).astype(np.complex64)
+        u, _, _, _ = _gpu(sssp, s, tl_every=0)
+        ref = _oracle(s, tl_every=steps)
+        err.append(np.linalg.norm(u - ref.u) / np.linalg.norm(ref.u))
+    assert np.mean(err) <= 7.85e-7, err
