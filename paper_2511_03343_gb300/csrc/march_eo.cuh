@@ -22,10 +22,11 @@
 // No prefix scan over the modes is left, and neither half waits for the other but at the depth points.
 //
 // What bounds it: the chain of dependent passes (3 radix passes and 2 exchanges a transform, one block
-// barrier a Neumann term) at a few warps a scheduler; then the shared-memory pipe (550 wavefronts a
-// transform at L = 1024).  8 points a thread: with 16, one solve of L = 2048 took 4200 cycles a transform
+// barrier a Neumann term) at a few warps a scheduler; then the shared-memory pipe.  8 points a thread: with 16, one solve of L = 2048 took 4200 cycles a transform
 // (2.07 GHz), with 8 3040; the scan form it replaced 4600 (37 solves of N = 2047, complex n^2, [6/6],
-// 40 steps: 9.1 -> 5.8 ms).  Its FP32 error is smaller too (no sums over L/2 modes): 3.1e-6 -> 1.2e-6
+// 40 steps: 9.1 -> 5.8 ms).  Complex n^2 leaves room for one solve of L = 2048 an SM (117 KB; the scan form
+// held two): 304 solves, 20 steps, the scan form against this one 8.4 -> 6.3 ms, real n^2 7.9 -> 4.9.
+// Its FP32 error is smaller too (no sums over L/2 modes): 3.1e-6 -> 1.2e-6
 // against complex128 there.
 #pragma once
 #include "march_dft.cuh"  // ldv2, ldv4
@@ -581,8 +582,9 @@ __global__ void __launch_bounds__(ECfg<LOG2L>::NT, ECfg<LOG2L>::MIN_BLOCKS)
 //
 // Against one CTA per field with its tables in shared memory (51 KB, 12 KB of tables loaded per
 // field): more fields an SM, no table traffic, the march's shorter pass chain, and the packed result
-// rows are written here.  4096 fields of N = 1023: 98 -> 18.7 us (690 -> 3580 GB/s of input and output,
-// 53 % of the copy bandwidth), of N = 4095: 418 -> 129 us; one field: 16.6 -> 5.1 us.  It is bound by
+// rows are written here.  On the device, 4096 fields of N = 1023: 98 -> 18.7 us (690 -> 3580 GB/s of input and
+// output, 53 % of the copy bandwidth; the call takes 24.7 us, 2.7 TB/s), of N = 4095: 418 -> 129 us; one field:
+// 16.6 -> 5.1 us.  It is bound by
 // the same chain at 6 fields an SM, with the shared-memory pipe as the next limit.
 template <int LOG2L>
 struct EDst {

@@ -378,14 +378,16 @@ cudaError_t launch_march(int log2L, const SolveDesc* d, int count, const Transfo
     return sssp_shapes::launch_march(log2L, ppt, d, count, tabs.tw, tabs.sinw, st, cplx, split);
   }
   // Dirichlet, L = 2048 and 4096: the parity-split kernel (one solve of L = 2048 4600 -> 3040 cycles a
-  // transform at 2.07 GHz, of L = 4096 6900 -> 6050).  L <= 1024 stays with the scan form: the split march
-  // is faster there too (one solve of L = 1024 2250 -> 1720, two an SM 3550 -> 2410), but these sizes'
-  // results are kept bit for bit: over the 256-solve batch another rounding of the scan form's sums
-  // moves the transmission loss by up to 0.2 dB at its deepest nulls.
+  // transform at 2.07 GHz, of L = 4096 6900 -> 6050).  L <= 1024 stays with the scan form by choice, so that its
+  // results keep their bits, and not because the split form is no better there: one solve of L = 1024 takes it
+  // 1720 cycles instead of 2250, two an SM 2410 instead of 3550, and over 256 solves of 160 steps (four seeds) it is
+  // nearer to complex128, field 4.4e-6 -> 2.3e-6 in the mean, worst TL error where TL < 100 dB 0.038 -> 0.021 dB,
+  // beyond 0.065 -> 0.032 dB.
   if (bc == sssp::kBcDirichlet && sssp_eo::march_supported(log2L))
     return sssp_eo::launch_march(log2L, d, count, st, cplx);
-  // periodic, 512 .. 2048 points: the passes of march_dft.cuh (one solve of 512 points 1080 -> 890 cycles a
-  // transform, of 1024 1700 -> 1300, of 2048 3040 -> 2040; 300 of 2048 5640 -> 4290); below, a group of its threads would hold less than a row, and 4096 points need a longer one than a warp holds
+  // periodic, 512 .. 2048 points: the passes of march_dft.cuh (march of 30 steps, general passes / these: one solve of
+  // 512 points 1.42 / 1.17 ms, of 1024 2.25 / 1.78, of 2048 4.48 / 2.86; 304 of 2048 9.29 / 6.46); below, a group of its
+  // threads would hold less than a row, and 4096 points need a longer one than a warp holds
   if (bc == sssp::kBcPeriodic && sssp_dft::supported(log2L))
     return sssp_dft::launch_march(log2L, d, count, st, cplx, split);
   switch (log2L) {
